@@ -100,11 +100,11 @@ def reference_model_bytes(n, s):
     return (2 * n0 * n1 * n2 + 24 * n0 * n1 * (n2 + 1) + (n0 + 1) * (n1 + 1) * (n2 + 1)) * s
 
 
-# Radix plan of the double-word (first-generation Stockham) line transforms,
-# per line length M = 2n; the same factorisation the kernels are built with.
-DW_RADICES = {8: [8], 12: [4, 3], 16: [4, 4], 24: [8, 3], 32: [8, 4], 48: [4, 4, 3], 64: [8, 8],
-              96: [8, 4, 3], 128: [8, 4, 4], 192: [8, 8, 3], 256: [8, 8, 4], 384: [8, 4, 4, 3],
-              512: [8, 8, 8], 768: [8, 8, 4, 3], 1024: [8, 8, 4, 4]}
+# Radix plan of the double-word Stockham line transforms, per line length
+# M = 2n; the same factorisation the kernels are built with (PlanDw).
+DW_RADICES = {8: [8], 12: [2, 3, 2], 16: [4, 4], 24: [2, 6, 2], 32: [4, 2, 4], 48: [4, 3, 4], 64: [8, 8],
+              96: [4, 6, 4], 128: [8, 2, 8], 192: [8, 3, 8], 256: [8, 4, 8], 384: [8, 6, 8],
+              512: [8, 8, 8], 768: [8, 3, 4, 8], 1024: [8, 4, 4, 8]}
 
 
 def dw_mid_ops(n):
@@ -112,7 +112,7 @@ def dw_mid_ops(n):
     is bound by the FP32 pipes, not by HBM).  Costs in FP32 operations: a
     double-word add 8 (TwoSum 6 + 2), multiply 6, complex add 16, complex
     twiddle product 32 (two fused dot products), complex scale 12.  Codelets:
-    DFT2/3/4/8 = 32/120/128/440; pruned first stage (zero upper half) of radix
+    DFT2/3/4/6/8 = 32/112/128/320/440; pruned first stage (zero upper half) of radix
     2/4/8 = 0/64/312; pruned last stage (lower half kept) = 16/96/376.  A
     column line (length M = 2 n1) is: forward transform (first stage pruned),
     multiply by the spectrum (M complex scales), inverse transform (last stage
@@ -123,7 +123,7 @@ def dw_mid_ops(n):
     n0, n1, n2 = n
     M = 2 * n1
     rad = DW_RADICES[M]
-    full = {2: 32, 3: 120, 4: 128, 8: 440}
+    full = {2: 32, 3: 112, 4: 128, 6: 320, 8: 440}
     half_in = {2: 0, 4: 64, 8: 312}
     half_out = {2: 16, 4: 96, 8: 376}
 

@@ -65,7 +65,6 @@ template <typename T> __device__ __forceinline__ T ddi_beta(const DdiPar* __rest
 // The pair of rho values the epilogue adds, as loaded (FP64 arrays for both
 // FP64 arithmetics).
 template <typename V> struct PairOf { using T = V; };
-template <> struct PairOf<cdw> { using T = double2; };
 
 template <typename V>
 __device__ __forceinline__ typename PairOf<V>::T load_rho_pair(const typename Io<V>::T* r) {
@@ -75,11 +74,7 @@ __device__ __forceinline__ typename PairOf<V>::T load_rho_pair(const typename Io
 template <typename V>
 __device__ __forceinline__ void store_pair_axpy(typename Io<V>::T* p, V v, typename Io<V>::T beta,
                                                 typename PairOf<V>::T a) {
-  if constexpr (std::is_same<V, cdw>::value) {
-    *reinterpret_cast<double2*>(p) = make_double2(dw_to_double(v.x) + beta * a.x, dw_to_double(v.y) + beta * a.y);
-  } else {
-    *reinterpret_cast<V*>(p) = mk(v.x + beta * a.x, v.y + beta * a.y);
-  }
+  *reinterpret_cast<V*>(p) = mk(v.x + beta * a.x, v.y + beta * a.y);
 }
 
 }  // namespace fsa

@@ -34,48 +34,20 @@ template <> struct RealOf<double2> { using T = double; };
 template <> struct RealOf<cdw> { using T = dw; };
 
 // Element types at the pass boundaries: T = the real type of rho and phi in
-// HBM, S = the stored spectrum's element type.  The double-word tier reads and
-// writes FP64 arrays and converts at the boundary.
+// HBM, S = the stored spectrum's element type.
 template <typename V> struct Io;
 template <> struct Io<float2> { using T = float; using S = float; };
 template <> struct Io<double2> { using T = double; using S = double; };
-template <> struct Io<cdw> { using T = double; using S = dw; };
 
 // two consecutive reals of rho as one complex value (a + i b)
 template <typename V> __device__ __forceinline__ V load_pair(const typename Io<V>::T* p) {
-  if constexpr (std::is_same<V, cdw>::value) {
-    const double2 d = *reinterpret_cast<const double2*>(p);
-    return mk(dw_from_double(d.x), dw_from_double(d.y));
-  } else {
-    return *reinterpret_cast<const V*>(p);
-  }
+  return *reinterpret_cast<const V*>(p);
 }
 template <typename V> __device__ __forceinline__ void store_pair(typename Io<V>::T* p, V v) {
-  if constexpr (std::is_same<V, cdw>::value) {
-    *reinterpret_cast<double2*>(p) = make_double2(dw_to_double(v.x), dw_to_double(v.y));
-  } else {
-    *reinterpret_cast<V*>(p) = v;
-  }
+  *reinterpret_cast<V*>(p) = v;
 }
 template <typename V> __device__ __forceinline__ typename RealOf<V>::T load_spec(const typename Io<V>::S* p) {
-  if constexpr (std::is_same<V, cdw>::value) {
-    const float2 f = __ldg(reinterpret_cast<const float2*>(p));
-    return dw(f.x, f.y);
-  } else {
-    return __ldg(p);
-  }
-}
-
-// Canonical form of a value leaving a pass for HBM.  The double-word
-// operations skip their closing renormalisation, so a low part can grow past
-// half an ulp of its high part over many operations; one TwoSum per part at
-// each pass boundary bounds that growth to the operations of one pass.
-template <typename V> __device__ __forceinline__ V canon(V v) {
-  if constexpr (std::is_same<V, cdw>::value) {
-    return mk(dw_two_sum(v.x.hi, v.x.lo), dw_two_sum(v.y.hi, v.y.lo));
-  } else {
-    return v;
-  }
+  return __ldg(p);
 }
 
 template <typename V> __device__ __forceinline__ V czero() { return mk(typename RealOf<V>::T(0), typename RealOf<V>::T(0)); }
@@ -87,13 +59,6 @@ template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
 // a * conj(b)
 template <typename V> __device__ __forceinline__ V cmulc(V a, V b) {
   return mk(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
-// double-word complex products: each part is one fused two-term dot product
-__device__ __forceinline__ cdw cmul(cdw a, cdw b) {
-  return mk(dw_dot2(a.x, b.x, -a.y, b.y), dw_dot2(a.x, b.y, a.y, b.x));
-}
-__device__ __forceinline__ cdw cmulc(cdw a, cdw b) {
-  return mk(dw_dot2(a.x, b.x, a.y, b.y), dw_dot2(a.y, b.x, -a.x, b.y));
 }
 template <typename V> __device__ __forceinline__ V cscale(V a, typename RealOf<V>::T s) { return mk(a.x * s, a.y * s); }
 
@@ -299,24 +264,18 @@ template <> struct PlanFor<1024> { using type = Plan<1024, 8, 8, 4, 4>; };
 // One copy per translation unit that includes this header.
 static __device__ float2 g_tw32[fsa::kTwN];
 static __device__ double2 g_tw64[fsa::kTwN];
-static __device__ fsa::cdw g_twdw[fsa::kTwN];
+static __device__ float4 g_twdw[fsa::kTwN];  // double-word: (re.hi, im.hi, re.lo, im.lo)
 
 namespace fsa {
 
 template <typename V> __device__ __forceinline__ const V* tw_table();
 template <> __device__ __forceinline__ const float2* tw_table<float2>() { return g_tw32; }
 template <> __device__ __forceinline__ const double2* tw_table<double2>() { return g_tw64; }
-template <> __device__ __forceinline__ const cdw* tw_table<cdw>() { return g_twdw; }
 
 // exp(-2 pi i e / L) for 0 <= e < L, L | 3072
 template <typename V, int L> __device__ __forceinline__ V twiddle(int e) {
   static_assert(kTwN % L == 0, "length must divide the twiddle table");
-  if constexpr (std::is_same<V, cdw>::value) {
-    const float4 f = __ldg(reinterpret_cast<const float4*>(tw_table<V>() + e * (kTwN / L)));
-    return mk(dw(f.x, f.y), dw(f.z, f.w));
-  } else {
-    return __ldg(tw_table<V>() + e * (kTwN / L));
-  }
+  return __ldg(tw_table<V>() + e * (kTwN / L));
 }
 
 // One Stockham stage S of plan P over a line, with T threads per line and

@@ -59,4 +59,55 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
   return true;
 }
 
+
+// Dynamic tiles: a kernel launched with one CTA per tile whose running CTAs
+// take over tiles not started yet (clusterlaunchcontrol, sm_100 and later),
+// so every SM keeps its full set of CTAs to the end.  (With a fixed share of
+// tiles per CTA the scheduler's favoured CTAs finish early: a double-word
+// middle pass ran at 23 of 32 resident warps on average.)  Thread 0 alone
+// asks and reads the answers; `next` publishes them to the CTA.
+struct TileQueue {
+  uint4 resp;                // the answer to the request in flight
+  unsigned long long bar;
+  int next;                  // the next tile, -1 = none
+  int pad;
+};
+static_assert(sizeof(TileQueue) == 32, "32 bytes of shared memory");
+__device__ __forceinline__ void tile_request(TileQueue* q) {  // thread 0
+  fence_proxy_async_smem();
+  mbar_arrive_expect_tx(&q->bar, 16);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];\n" ::"r"(
+                   smem_u32(&q->resp)),
+               "r"(smem_u32(&q->bar))
+               : "memory");
+}
+// thread 0, before the CTA's first barrier: the first request
+__device__ __forceinline__ void tile_queue_init(TileQueue* q) {
+  mbar_init(&q->bar, 1);
+  fence_mbar_init();
+  q->next = -1;
+  tile_request(q);
+}
+// thread 0: wait (bounded) for the answer to the request in flight and
+// publish it (read `next` after a barrier).  A wait that gives up ends this
+// CTA's tiles and is recorded in the fault word.
+__device__ __forceinline__ void tile_answer(TileQueue* q, unsigned parity, unsigned int* fault) {
+  int next = -1;
+  if (mbar_wait(&q->bar, parity)) {
+    unsigned ok, x;
+    asm volatile(
+        "{\n .reg .b128 r;\n .reg .pred p;\n ld.shared.b128 r, [%2];\n"
+        " clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n selp.u32 %0, 1, 0, p;\n mov.u32 %1, 0;\n"
+        " @p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n}\n"
+        : "=r"(ok), "=r"(x)
+        : "r"(smem_u32(&q->resp))
+        : "memory");
+    if (ok) next = (int)x;
+  } else {
+    if (fault) atomicOr(fault, kWaitTimeout);
+    mbar_wait(&q->bar, parity);  // the answer still in flight
+  }
+  q->next = next;
+}
+
 }  // namespace fsa

@@ -34,23 +34,6 @@ namespace fsa {
 
 template <typename V> struct TileW { static constexpr int W = 16; };
 template <> struct TileW<double2> { static constexpr int W = 8; };
-template <> struct TileW<cdw> { static constexpr int W = 4; };
-
-// Resident CTAs per SM the compiler should allow for: double-word passes are
-// bound by the FP32 pipes; they run 4-line tiles (256 threads for length
-// 512) four to an SM (at most 64 registers), so a barrier holds fewer warps
-// (R2C 0.218 against 0.255 ms, C2R 0.204 against 0.230 ms at 256^3 with
-// 8-line tiles two to an SM; the row passes the same).
-template <typename V> struct MinB { static constexpr int value = 1; };
-template <> struct MinB<cdw> { static constexpr int value = 4; };
-
-// The middle pass keeps a whole line's forward transform, multiply and
-// inverse in one CTA; for double-word values it takes half-width tiles so
-// that two CTAs (each up to 128 registers a thread) share an SM and one's
-// barriers and loads overlap the other's arithmetic.
-template <typename V> struct MidW { static constexpr int W = TileW<V>::W; };
-template <> struct MidW<cdw> { static constexpr int W = 4; };
-template <typename V, int NT> constexpr int minb_mid() { return (std::is_same<V, cdw>::value && NT <= 256) ? 2 : 1; }
 
 // Threads per line: one butterfly of the largest radix per thread, capped so
 // that a CTA has at most 512 threads.
@@ -70,7 +53,7 @@ template <class P, typename V, int W> constexpr int smem_rows() { return W * (P:
 // PAD = false: the unpadded transform of length M over all M inputs (the DDI
 // grid reading's derivative, Sec. 5 Example 4); the same K = M/2 + 1 outputs.
 template <typename V, class P, int W, int T, bool PAD = true>
-__global__ void __launch_bounds__(W * T, MinB<V>::value) k_r2c_ax0(const Jobs jobs, long long C) {
+__global__ void __launch_bounds__(W * T) k_r2c_ax0(const Jobs jobs, long long C) {
   using R = typename RealOf<V>::T;
   constexpr int M = P::M, NV = PAD ? M / 2 : M, K = M / 2 + 1;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -96,8 +79,8 @@ __global__ void __launch_bounds__(W * T, MinB<V>::value) k_r2c_ax0(const Jobs jo
     const V a = mk(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
     const V b = mk(R(0.5) * (zk.y + zm.y), R(0.5) * (zm.x - zk.x));
     if (ok) {
-      X[(long long)k * C + c] = canon(a);
-      X[(long long)k * C + c + 1] = canon(b);
+      X[(long long)k * C + c] = a;
+      X[(long long)k * C + c + 1] = b;
     }
   }
   __syncthreads();
@@ -106,7 +89,7 @@ __global__ void __launch_bounds__(W * T, MinB<V>::value) k_r2c_ax0(const Jobs jo
 
 // ---------------------------------------------------------------- pass 2 --
 template <typename V, class P, int W, int T, bool PAD = true>
-__global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_fwd(const Jobs jobs, long long rows) {
+__global__ void __launch_bounds__(W * T) k_row_fwd(const Jobs jobs, long long rows) {
   constexpr int M = P::M, n = PAD ? M / 2 : M, PITCH = M + 1, NT = W * T;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
@@ -130,7 +113,7 @@ __global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_fwd(const Jobs jo
   for (int i = threadIdx.x; i < W * M; i += NT) {
     const int l2 = i / M, p = i - l2 * M;
     const long long row = row0 + l2;
-    if (row < rows) Y[row * M + p] = canon(sm[l2 * PITCH + p]);
+    if (row < rows) Y[row * M + p] = sm[l2 * PITCH + p];
   }
   __syncthreads();
   }
@@ -141,7 +124,7 @@ __global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_fwd(const Jobs jo
 // modes by the multiplier of jb.par, kMulDdiGrid on the unpadded grid (all
 // M entries of a column live, transform length M along every axis).
 template <typename V, class P, int W, int T, int MODE = kMulSpectrum>
-__global__ void __launch_bounds__(W * T, minb_mid<V, W * T>()) k_col_mid(const Jobs jobs, int M2, int planes) {
+__global__ void __launch_bounds__(W * T) k_col_mid(const Jobs jobs, int M2, int planes) {
   using R = typename RealOf<V>::T;
   constexpr bool PAD = MODE != kMulDdiGrid;
   constexpr int M = P::M, n = PAD ? M / 2 : M;
@@ -177,7 +160,7 @@ __global__ void __launch_bounds__(W * T, minb_mid<V, W * T>()) k_col_mid(const J
     return cscale(sl.get(p), s);
   };
   auto last = [&](int p, V v) {
-    if (p < n && ok) col[(long long)p * M2] = canon(v);
+    if (p < n && ok) col[(long long)p * M2] = v;
   };
   fft_line<P, false, T, V, false, PAD>(t, mul, last, sl);
   }
@@ -190,7 +173,7 @@ __global__ void __launch_bounds__(W * T, minb_mid<V, W * T>()) k_col_mid(const J
 // even; row stride n1 + 1), transformed back and cropped to n1 values, in
 // place.  W rows per CTA in an odd-pitch shared tile, as the row passes.
 template <typename V, class P, int W, int T>
-__global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_mid(const Jobs jobs, long long rows) {
+__global__ void __launch_bounds__(W * T) k_row_mid(const Jobs jobs, long long rows) {
   using R = typename RealOf<V>::T;
   constexpr int M = P::M, n = M / 2, PITCH = M + 1, NT = W * T;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -223,7 +206,7 @@ __global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_mid(const Jobs jo
   for (int i = threadIdx.x; i < W * n; i += NT) {
     const int l2 = i / n, p = i - l2 * n;
     const long long r2 = row0 + l2;
-    if (r2 < rows) X[r2 * n + p] = canon(sm[l2 * PITCH + p]);
+    if (r2 < rows) X[r2 * n + p] = sm[l2 * PITCH + p];
   }
   __syncthreads();
   }
@@ -231,7 +214,7 @@ __global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_mid(const Jobs jo
 
 // ---------------------------------------------------------------- pass 4 --
 template <typename V, class P, int W, int T, bool PAD = true>
-__global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_inv(const Jobs jobs, long long rows) {
+__global__ void __launch_bounds__(W * T) k_row_inv(const Jobs jobs, long long rows) {
   constexpr int M = P::M, n = PAD ? M / 2 : M, PITCH = M + 1, NT = W * T;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
@@ -255,7 +238,7 @@ __global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_inv(const Jobs jo
   for (int i = threadIdx.x; i < W * n; i += NT) {
     const int l2 = i / n, p = i - l2 * n;
     const long long row = row0 + l2;
-    if (row < rows) X[row * n + p] = canon(sm[l2 * PITCH + p]);
+    if (row < rows) X[row * n + p] = sm[l2 * PITCH + p];
   }
   __syncthreads();
   }
@@ -265,7 +248,7 @@ __global__ void __launch_bounds__(W * T, MinB<V>::value) k_row_inv(const Jobs jo
 // EPI: the output is phi + beta * rho with rho = jb.aux, beta = the DDI block's kDdiBeta
 // (the DDI grid reading's local term).
 template <typename V, class P, int W, int T, bool PAD = true, bool EPI = false>
-__global__ void __launch_bounds__(W * T, MinB<V>::value) k_c2r_ax0(const Jobs jobs, long long C) {
+__global__ void __launch_bounds__(W * T) k_c2r_ax0(const Jobs jobs, long long C) {
   using R = typename RealOf<V>::T;
   constexpr int M = P::M, n = M / 2, NV = PAD ? M / 2 : M;
   extern __shared__ __align__(16) unsigned char smraw[];

@@ -23,10 +23,6 @@ template <typename V, int M> struct Inst {
   static constexpr int NT = W * T;
   static constexpr int SM_STRIDED = smem_strided<P, V, W>();
   static constexpr int SM_ROWS = smem_rows<P, V, W>();
-  static constexpr int WC = MidW<V>::W;  // middle pass tile
-  static constexpr int TC = threads_per_line<P, WC>();
-  static constexpr int NTC = WC * TC;
-  static constexpr int SM_MID = smem_strided<P, V, WC>();
 
   static cudaError_t prepare() {
     cudaError_t e = cudaSuccess;
@@ -35,18 +31,18 @@ template <typename V, int M> struct Inst {
     };
     set((const void*)k_r2c_ax0<V, P, W, T>, SM_STRIDED);
     set((const void*)k_row_fwd<V, P, W, T>, SM_ROWS);
-    set((const void*)k_col_mid<V, P, WC, TC>, SM_MID);
+    set((const void*)k_col_mid<V, P, W, T>, SM_STRIDED);
     set((const void*)k_row_inv<V, P, W, T>, SM_ROWS);
     set((const void*)k_row_mid<V, P, WM, TM>, SM_ROWM);
     set((const void*)k_r2c_ax0<V, P, WM, TM>, SM_STRM);
     set((const void*)k_c2r_ax0<V, P, WM, TM>, SM_STRM);
     set((const void*)k_c2r_ax0<V, P, W, T>, SM_STRIDED);
-    set((const void*)k_col_mid<V, P, WC, TC, kMulDdiKernel>, SM_MID);
+    set((const void*)k_col_mid<V, P, W, T, kMulDdiKernel>, SM_STRIDED);
     set((const void*)k_c2r_ax0<V, P, W, T, true, true>, SM_STRIDED);
     if constexpr (kUnpadded) {
       set((const void*)k_r2c_ax0<V, P, W, T, false>, SM_STRIDED);
       set((const void*)k_row_fwd<V, P, W, T, false>, SM_ROWS);
-      set((const void*)k_col_mid<V, P, WC, TC, kMulDdiGrid>, SM_MID);
+      set((const void*)k_col_mid<V, P, W, T, kMulDdiGrid>, SM_STRIDED);
       set((const void*)k_row_inv<V, P, W, T, false>, SM_ROWS);
       set((const void*)k_c2r_ax0<V, P, W, T, false>, SM_STRIDED);
     }
@@ -54,9 +50,9 @@ template <typename V, int M> struct Inst {
   }
   static Geometry geometry(PassKind k) {
     Geometry g;
-    g.W = k == kColMid ? WC : W;
-    g.threads = k == kColMid ? NTC : NT;
-    g.smem = (k == kRowFwd || k == kRowInv) ? SM_ROWS : (k == kColMid ? SM_MID : SM_STRIDED);
+    g.W = W;
+    g.threads = NT;
+    g.smem = (k == kRowFwd || k == kRowInv) ? SM_ROWS : SM_STRIDED;
     return g;
   }
   static cudaError_t r2c(const Jobs& jobs, long long C, cudaStream_t s) {
@@ -72,9 +68,9 @@ template <typename V, int M> struct Inst {
     return cudaGetLastError();
   }
   static cudaError_t colm(const Jobs& jobs, int M2, int planes, cudaStream_t s) {
-    const long long tiles = (long long)((M2 + WC - 1) / WC) * planes * jobs.count;
-    auto f = k_col_mid<V, P, WC, TC>;
-    f<<<persistent_grid((const void*)f, NTC, SM_MID, tiles), NTC, SM_MID, s>>>(jobs, M2, planes);
+    const long long tiles = (long long)((M2 + W - 1) / W) * planes * jobs.count;
+    auto f = k_col_mid<V, P, W, T>;
+    f<<<persistent_grid((const void*)f, NT, SM_STRIDED, tiles), NT, SM_STRIDED, s>>>(jobs, M2, planes);
     return cudaGetLastError();
   }
   // the d = 2 middle pass: rows of the R2C output, in place.  A plane has
@@ -123,9 +119,9 @@ template <typename V, int M> struct Inst {
   // (this instance's length is the grid's n there) whose middle multiplies by
   // cmul * D.
   static cudaError_t colm_ddi(const Jobs& jobs, int M2, int planes, cudaStream_t s) {
-    const long long tiles = (long long)((M2 + WC - 1) / WC) * planes * jobs.count;
-    auto f = k_col_mid<V, P, WC, TC, kMulDdiKernel>;
-    f<<<persistent_grid((const void*)f, NTC, SM_MID, tiles), NTC, SM_MID, s>>>(jobs, M2, planes);
+    const long long tiles = (long long)((M2 + W - 1) / W) * planes * jobs.count;
+    auto f = k_col_mid<V, P, W, T, kMulDdiKernel>;
+    f<<<persistent_grid((const void*)f, NT, SM_STRIDED, tiles), NT, SM_STRIDED, s>>>(jobs, M2, planes);
     return cudaGetLastError();
   }
   static cudaError_t c2r_epi(const Jobs& jobs, long long C, cudaStream_t s) {
@@ -147,9 +143,9 @@ template <typename V, int M> struct Inst {
     return cudaGetLastError();
   }
   static cudaError_t colm_per(const Jobs& jobs, int M2, int planes, cudaStream_t s) {
-    const long long tiles = (long long)((M2 + WC - 1) / WC) * planes * jobs.count;
-    auto f = k_col_mid<V, P, WC, TC, kMulDdiGrid>;
-    f<<<persistent_grid((const void*)f, NTC, SM_MID, tiles), NTC, SM_MID, s>>>(jobs, M2, planes);
+    const long long tiles = (long long)((M2 + W - 1) / W) * planes * jobs.count;
+    auto f = k_col_mid<V, P, W, T, kMulDdiGrid>;
+    f<<<persistent_grid((const void*)f, NT, SM_STRIDED, tiles), NT, SM_STRIDED, s>>>(jobs, M2, planes);
     return cudaGetLastError();
   }
   static cudaError_t rowi_per(const Jobs& jobs, long long rows, cudaStream_t s) {
@@ -402,15 +398,16 @@ static cudaError_t init_tu_twiddles() {
   host_twiddles(re.data(), im.data());
   std::vector<float2> t32(kTwN);
   std::vector<double2> t64(kTwN);
-  std::vector<cdw> tdw(kTwN);
+  std::vector<float4> tdw(kTwN);  // (re.hi, im.hi, re.lo, im.lo)
   for (int k = 0; k < kTwN; ++k) {
     t32[k] = make_float2((float)re[k], (float)im[k]);
     t64[k] = make_double2(re[k], im[k]);
-    tdw[k] = cdw{dw(re[k]), dw(im[k])};
+    const dw c(re[k]), s(im[k]);
+    tdw[k] = make_float4(c.hi, s.hi, c.lo, s.lo);
   }
   cudaError_t e = cudaMemcpyToSymbol(g_tw32, t32.data(), sizeof(float2) * kTwN);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_tw64, t64.data(), sizeof(double2) * kTwN);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_twdw, tdw.data(), sizeof(cdw) * kTwN);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_twdw, tdw.data(), sizeof(float4) * kTwN);
   return e;
 }
 
