@@ -208,10 +208,13 @@ cudaError_t tensorgen_prepare(int M);
 // which must be current; once per device (noalloc.cu).
 cudaError_t noalloc_resolve(int dev);
 cudaError_t tensorgen_init_twiddles();
-// param: the kernel's parameter (the Yukawa lam), ignored by the others
+// param: the kernel's parameter (the Yukawa lam), ignored by the others.
+// utab_mem, wtab_mem: room for a quarter of the octant's points in doubles
+// each (tables of U^eps and W, used until the call's work ends), or null.
 cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], double eps, double param,
                           double* oct64, void* out, fsa_dtype dtype, cudaStream_t s,
-                          const double* wtab = nullptr, int wtab_panels = 0);
+                          const double* wtab = nullptr, int wtab_panels = 0, double* utab_mem = nullptr,
+                          double* wtab_mem = nullptr);
 
 // Twiddle table exp(-2 pi i k / 3072), k < 3072, computed on the host.
 void host_twiddles(double* re, double* im);

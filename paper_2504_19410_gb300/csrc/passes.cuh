@@ -1,5 +1,5 @@
-// The five apply passes of the pruned zero-padded 3-D convolution and the
-// DCT-I pass of tensor generation, as templates over the complex type
+// The five apply passes of the pruned zero-padded 3-D convolution, as
+// templates over the complex type
 // (float2 / double2), the transform plan (length M = 2n) and the tile shape
 // (W lines per CTA, T threads per line).
 //
@@ -303,38 +303,6 @@ __global__ void __launch_bounds__(W * T) k_c2r_ax0(const Jobs jobs, long long C)
     __syncthreads();
   }
   }
-}
-
-// ------------------------------------------------------------- DCT-I pass --
-// In place on an FP64 array: for each line (n+1 values O[0..n] with element
-// stride es), O[p] <- O[0] + (-1)^p O[n] + 2 sum_{j=1}^{n-1} O[j] cos(pi j p / n),
-// i.e. the length-2n DFT of the even extension O[min(m, 2n-m)].  Two lines
-// ride in one complex transform (their DFTs are real, so they come back as
-// the real and imaginary parts).  Line L starts at (L / inner) * os + (L % inner) * is.
-template <class P, int W, int T>
-__global__ void __launch_bounds__(W * T) k_dct1(double* __restrict__ O, long long nlines, long long inner,
-                                                long long os, long long is, long long es) {
-  constexpr int M = P::M, n = M / 2;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  double2* sm = reinterpret_cast<double2*>(smraw);
-  const int l = threadIdx.x % W, t = threadIdx.x / W;
-  const long long q = (long long)blockIdx.x * W + l;
-  const long long L0 = 2 * q, L1 = 2 * q + 1;
-  const bool ok0 = L0 < nlines, ok1 = L1 < nlines;
-  const long long b0 = ok0 ? (L0 / inner) * os + (L0 % inner) * is : 0;
-  const long long b1 = ok1 ? (L1 / inner) * os + (L1 % inner) * is : 0;
-  SLine<double2, W> sl{sm + l};
-  auto first = [&](int m) -> double2 {
-    const long long mm = m <= n ? m : M - m;
-    return mk(ok0 ? O[b0 + mm * es] : 0.0, ok1 ? O[b1 + mm * es] : 0.0);
-  };
-  auto last = [&](int p, double2 v) {
-    if (p <= n) {
-      if (ok0) O[b0 + p * es] = v.x;
-      if (ok1) O[b1 + p * es] = v.y;
-    }
-  };
-  fft_line<P, true, T, double2>(t, first, last, sl);
 }
 
 }  // namespace fsa

@@ -1217,12 +1217,28 @@ fsa_status attach_w_table(fsa_plan* p) {
   return FSA_OK;
 }
 
-cudaError_t plan_generate_into(fsa_plan* p, void* scratch, cudaStream_t s) {
+// scratch, scratch_bytes: FP32 plans: at least plan_gen_scratch_bytes.  The
+// radial tables (tensor_gen.cu) take memory the generation does not use
+// otherwise: FP64 plans the double-word copy's, before it is made; FP32 plans
+// the spectrum's for U^eps (written only by the last pass) and, for W, what the
+// scratch holds beyond the octant (a plan's workspace does; a serving plan's
+// scratch does not, and evaluates W per point).
+cudaError_t plan_generate_into(fsa_plan* p, void* scratch, size_t scratch_bytes, cudaStream_t s) {
   double* oct = p->dtype == FSA_F64 ? (double*)p->spectrum : (double*)scratch;
+  const size_t total = octant_count(p->n, p->d), quarter = align256(total / 4 * 8);
+  double *ut = nullptr, *wt = nullptr;
+  if (p->dtype == FSA_F64 && p->spectrum_dw) {
+    ut = (double*)p->spectrum_dw;
+    if (2 * quarter <= total * 8) wt = (double*)((char*)p->spectrum_dw + quarter);
+  } else if (p->dtype == FSA_F32) {
+    ut = (double*)p->spectrum;
+    const size_t off = align256(total * 8);
+    if (scratch_bytes >= off + quarter) wt = (double*)((char*)scratch + off);
+  }
   // a DDI plan's tensor is the Coulomb kernel's (Sec. 5, Example 4)
   const fsa_kernel k = p->kernel == FSA_KERNEL_DDI3D ? FSA_KERNEL_COULOMB3D : p->kernel;
   cudaError_t e = tensorgen_run(k, p->n, p->L, p->eps, p->param, oct, p->spectrum, p->dtype, s, p->wtab,
-                                p->wtab_panels);
+                                p->wtab_panels, ut, wt);
   if (e == cudaSuccess && p->spectrum_dw)
     e = spectrum_to_dw((const double*)p->spectrum, p->spectrum_dw, p->spectrum_bytes / 8, s);
   if (e == cudaSuccess) p->generated = 1;
@@ -1419,7 +1435,7 @@ fsa_status fsa_tensor_generate(fsa_plan* p, fsa_stream_t stream) {
   if (e != cudaSuccess) return cuda_error(e, "fsa_tensor_generate: cudaSetDevice");
   if (!p->ws && p->dtype == FSA_F32)
     return set_error(FSA_ERR_INVALID_ARG, "fsa_tensor_generate: plan has no workspace for its FP64 scratch");
-  e = plan_generate_into(p, p->ws, (cudaStream_t)stream);
+  e = plan_generate_into(p, p->ws, p->ws_bytes, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_error(e, "fsa_tensor_generate: launch");
   return FSA_OK;
 }

@@ -36,7 +36,7 @@
 namespace fsa {
 fsa_status plan_create_internal(fsa_plan** out, fsa_kernel kernel, const double* L, const int* n, fsa_dtype dtype,
                                 double eps, double eps_tol, bool with_workspace, double param);
-cudaError_t plan_generate_into(fsa_plan* p, void* scratch, cudaStream_t s);
+cudaError_t plan_generate_into(fsa_plan* p, void* scratch, size_t scratch_bytes, cudaStream_t s);
 size_t plan_workspace_bytes(const int* n, fsa_dtype dt);
 size_t plan_gen_scratch_bytes(const int* n, fsa_dtype dt, int d);
 size_t plan_resident_bytes(const int* n, fsa_dtype dt, int d);
@@ -236,7 +236,7 @@ bool try_admit(fsa_server* s, uint64_t id) {
       void* scratch = nullptr;
       cudaEvent_t ready = nullptr;
       if (gen_scratch) e = cudaMallocFromPoolAsync(&scratch, gen_scratch, s->pool, stream);
-      if (e == cudaSuccess) e = plan_generate_into(p, scratch, stream);
+      if (e == cudaSuccess) e = plan_generate_into(p, scratch, gen_scratch, stream);
       if (scratch) cudaFreeAsync(scratch, stream);
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
       if (e == cudaSuccess) e = cudaEventRecord(ready, stream);

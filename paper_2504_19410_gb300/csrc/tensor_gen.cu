@@ -38,12 +38,24 @@
 //     (d = 2 everywhere, d = 3 near r = 0 where the closed form cancels) the
 //     integral in x = ln(4t/eps^2) by composite 16-point Gauss-Legendre
 //     quadrature on panels of width 1/2 up to where exp(-lam^2 t) < e^-60.
+//
+// T^(1) and W are radial, and on the octant their arguments are
+// r = b sqrt(q), k = c sqrt(q') with q = sum_j r_j p_j^2 an integer wherever the
+// mesh steps' (the box's) squared ratios are: a cube of 256^3 has 17.0e6
+// points but only 196,609 values of q.  Both functions are then tabulated over
+// q (k_radial_tables) and looked up by the first and the last DCT pass, which
+// saves their per-point evaluation on the FP64 pipe and three passes over
+// the octant.  Measured (GB300, FP64 plan of 256^3): octant
+// 2.60 and spectrum 0.89 ms before, 0.05 ms for the tables now; with the
+// pruned DCT passes the whole generation 6.65 -> 2.00 ms.
+// Other grids (no common integer ratio, or a table above a quarter of the
+// octant: planes, very flat boxes) evaluate per point.
 #include <algorithm>
 #include <cmath>
 #include <vector>
 
+#include "dct.cuh"
 #include "fsa_internal.h"
-#include "passes.cuh"
 #include "quad.h"
 
 namespace fsa {
@@ -209,6 +221,34 @@ __global__ void k_t1_octant(double* __restrict__ O, int kernel, int n0, int n1, 
   }
 }
 
+// u[q] = hv U^eps(b sqrt(q)) for q < nu, w[q] = W(c sqrt(q)) for q < nw.  All
+// points of one q share its rounding error, which the DCT would then average
+// less than per-point errors; so for the 3-D Coulomb kernel the algebraic part
+// f / sqrt(q), f = hv / (4 pi b) = fh + fl, is formed to twice the working
+// precision and rounded once.
+__device__ double w_from_table(const double* __restrict__ tab, int P, double k);
+__global__ void k_radial_tables(double* __restrict__ u, long long nu, double b, double hv, double fh, double fl,
+                                double* __restrict__ w,
+                                long long nw, double c, int kernel, double eps, double lam,
+                                const double* __restrict__ wtab, int wpanels) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nu + nw;
+       i += (long long)gridDim.x * blockDim.x) {
+    if (i < nu) {
+      const double s = sqrt((double)i);
+      if (kernel == FSA_KERNEL_COULOMB3D && i > 0) {
+        const double ds = fma(-s, s, (double)i) / (2.0 * s);  // sqrt(i) = s + ds
+        const double t = fh / s;
+        u[i] = erf(b * s / eps) * (t + (fma(-t, s, fh) + (fl - t * ds)) / s);
+      } else {
+        u[i] = hv * smooth_U(kernel, b * s, eps, lam);
+      }
+    } else {
+      const double q = (double)(i - nu);
+      w[i - nu] = wtab ? w_from_table(wtab, wpanels, c * sqrt(q)) : singular_W(kernel, c * c * q, eps * eps, lam);
+    }
+  }
+}
+
 // W(k) from the quadrature table of radial_w.cpp: the panel holding k (binary
 // search over the edges), then its Chebyshev series by Clenshaw's recurrence.
 __device__ double w_from_table(const double* __restrict__ tab, int P, double k) {
@@ -268,19 +308,27 @@ cudaError_t spectrum_to_dw(const double* src, void* dst, size_t count, cudaStrea
 
 namespace {
 
+// One DCT pass: the octant in place, from the U table, or to the spectrum.
 template <int M> struct DctInst {
   using P = typename PlanFor<M>::type;
   static constexpr int W = 8;
   static constexpr int T = threads_per_line<P, W>();
   static constexpr int SM = smem_strided<P, double2, W>();
-  static cudaError_t prepare() {
-    return cudaFuncSetAttribute((const void*)k_dct1<P, W, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
+  template <class Src, class Dst> static cudaError_t set() {
+    return cudaFuncSetAttribute((const void*)k_dct1<P, W, T, Src, Dst>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
   }
-  static cudaError_t run(double* O, long long nlines, long long inner, long long os, long long is, long long es,
-                         cudaStream_t s) {
+  static cudaError_t prepare() {
+    cudaError_t e = set<DctArray, DctArray>();
+    if (e == cudaSuccess) e = set<DctRadial, DctArray>();
+    if (e == cudaSuccess) e = set<DctArray, DctSpectrum<float>>();
+    if (e == cudaSuccess) e = set<DctArray, DctSpectrum<double>>();
+    return e;
+  }
+  template <class Src, class Dst>
+  static cudaError_t run(const Src& src, const Dst& dst, long long nlines, int inner, cudaStream_t s) {
     const long long pairs = (nlines + 1) / 2;
     const long long tiles = (pairs + W - 1) / W;
-    k_dct1<P, W, T><<<(unsigned)tiles, W * T, SM, s>>>(O, nlines, inner, os, is, es);
+    k_dct1<P, W, T><<<(unsigned)tiles, W * T, SM, s>>>(src, dst, nlines, inner);
     return cudaGetLastError();
   }
 };
@@ -310,13 +358,44 @@ cudaError_t dct_prepare(int M) {
   return cudaErrorInvalidValue;
 }
 
-cudaError_t dct_run(int M, double* O, long long nlines, long long inner, long long os, long long is, long long es,
-                    cudaStream_t s) {
-  FSA_DCT_DISPATCH(M, run(O, nlines, inner, os, is, es, s));
+template <class Src, class Dst>
+cudaError_t dct_run(int M, const Src& src, const Dst& dst, long long nlines, long long inner, cudaStream_t s) {
+  FSA_DCT_DISPATCH(M, run(src, dst, nlines, (int)inner, s));
   return cudaErrorInvalidValue;
 }
 
 #undef FSA_DCT_DISPATCH
+
+// The integers r_j with s_j^2 = base^2 r_j (to round-off) and the table length
+// sum_j r_j n_j^2 + 1; false where no base s_min / m, m <= 3, gives integers or
+// the table would hold more than a quarter of the octant's points (more
+// evaluations saved than made, and room for two tables in the octant).
+struct Radial {
+  double base;
+  int r[3];
+  long long size;
+};
+bool radial_of(const double* sj, const int* n, long long total, Radial* out) {
+  const double lo = std::min(sj[0], std::min(sj[1], sj[2]));
+  for (int m = 1; m <= 3; ++m) {
+    out->base = lo / m;
+    long long size = 1;
+    bool ok = true;
+    for (int j = 0; j < 3 && ok; ++j) {
+      const double x = sj[j] / lo, v = x * x * (m * m), rv = std::nearbyint(v);
+      ok = std::fabs(v - rv) <= 4e-15 * rv && rv * n[j] * n[j] < 1e9;
+      if (ok) {
+        out->r[j] = (int)rv;
+        size += (long long)rv * n[j] * n[j];
+      }
+    }
+    if (ok && size <= total / 4) {
+      out->size = size;
+      return true;
+    }
+  }
+  return false;
+}
 
 }  // namespace
 
@@ -341,7 +420,8 @@ cudaError_t tensorgen_init_twiddles() {
 }
 
 cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], double eps, double lam, double* O,
-                          void* out, fsa_dtype dtype, cudaStream_t s, const double* wtab, int wtab_panels) {
+                          void* out, fsa_dtype dtype, cudaStream_t s, const double* wtab, int wtab_panels,
+                          double* utab_mem, double* wtab_mem) {
   // d = 2: a single plane of the octant (n2 = 0 here, unit h2), no axis-2 DCT
   const bool plane = kernel_dim(kernel) == 2;
   const int n0 = n[0], n1 = n[1], n2 = plane ? 0 : n[2];
@@ -349,27 +429,51 @@ cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], 
   const double h0 = 2.0 * L[0] / n0, h1 = 2.0 * L[1] / n1, h2 = plane ? 1.0 : 2.0 * L[2] / n2;
   const long long total = e0 * e1 * e2;
   const int threads = 256;
-  const int blocks = (int)std::min<long long>((total + threads - 1) / threads, 152LL * 16);
-  k_t1_octant<<<blocks, threads, 0, s>>>(O, (int)kernel, n0, n1, n2, h0, h1, h2, eps, lam);
-  cudaError_t e = cudaGetLastError();
-  // axis 2: lines (p0, p1) contiguous, element stride 1
-  if (e == cudaSuccess && !plane) e = dct_run(2 * n2, O, e0 * e1, e1, e1 * e2, e2, 1, s);
-  // axis 1: lines (p0, p2), element stride e2
-  if (e == cudaSuccess) e = dct_run(2 * n1, O, e0 * e2, e2, e1 * e2, 1, e2, s);
-  // axis 0: lines (p1, p2) flattened, element stride e1 * e2
-  if (e == cudaSuccess) e = dct_run(2 * n0, O, e1 * e2, e1 * e2, 0, 1, e1 * e2, s);
-  if (e != cudaSuccess) return e;
+  const auto blocks_for = [&](long long count) {
+    return (int)std::min<long long>((count + threads - 1) / threads, 152LL * 16);
+  };
   const double pi = 3.14159265358979323846;
   const double inv_norm = plane ? 1.0 / (4.0 * (double)n0 * n1) : 1.0 / (8.0 * (double)n0 * n1 * n2);
   const double c2 = plane ? 0.0 : pi / (2 * L[2]);
+  const double hs[3] = {h0, h1, h2}, cs[3] = {pi / (2 * L[0]), pi / (2 * L[1]), c2};
+  Radial ru{}, rw{};
+  const bool tu = !plane && utab_mem && radial_of(hs, n, total, &ru);
+  const bool tw = !plane && wtab_mem && radial_of(cs, n, total, &rw);
+  cudaError_t e = cudaSuccess;
+  if (tu || tw) {
+    const long long nu = tu ? ru.size : 0, nw = tw ? rw.size : 0;
+    const long double f = (long double)h0 * h1 * h2 / (4.0L * 3.141592653589793238462643383279502884L * ru.base);
+    const double fh = tu ? (double)f : 0.0, fl = tu ? (double)(f - (long double)fh) : 0.0;
+    k_radial_tables<<<blocks_for(nu + nw), threads, 0, s>>>(utab_mem, nu, ru.base, h0 * h1 * h2, fh, fl, wtab_mem, nw,
+                                                            rw.base, (int)kernel, eps, lam, wtab, wtab_panels);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess && !tu) {
+    k_t1_octant<<<blocks_for(total), threads, 0, s>>>(O, (int)kernel, n0, n1, n2, h0, h1, h2, eps, lam);
+    e = cudaGetLastError();
+  }
+  // axis 2: lines (p0, p1), element stride 1
+  const DctArray x2{O, e1 * e2, e2, 1};
+  if (e == cudaSuccess && !plane)
+    e = tu ? dct_run(2 * n2, DctRadial{utab_mem, ru.r[0], ru.r[1], ru.r[2]}, x2, e0 * e1, e1, s)
+           : dct_run(2 * n2, x2, x2, e0 * e1, e1, s);
+  // axis 1: lines (p0, p2), element stride e2
+  const DctArray x1{O, e1 * e2, 1, e2};
+  if (e == cudaSuccess) e = dct_run(2 * n1, x1, x1, e0 * e2, e2, s);
+  // axis 0: lines (p1, p2), element stride e1 * e2
+  const DctArray x0{O, e2, 1, e1 * e2};
+  const DctRadial w0{wtab_mem, rw.r[1], rw.r[2], rw.r[0]};
+  if (e == cudaSuccess)
+    e = !tw                  ? dct_run(2 * n0, x0, x0, e1 * e2, e2, s)
+        : dtype == FSA_F64 ? dct_run(2 * n0, x0, DctSpectrum<double>{(double*)out, x0, w0, inv_norm}, e1 * e2, e2, s)
+                           : dct_run(2 * n0, x0, DctSpectrum<float>{(float*)out, x0, w0, inv_norm}, e1 * e2, e2, s);
+  if (e != cudaSuccess || tw) return e;
   if (dtype == FSA_F64)
-    k_spectrum_finalize<double><<<blocks, threads, 0, s>>>(O, (double*)out, (int)kernel, n0, n1, n2, pi / (2 * L[0]),
-                                                           pi / (2 * L[1]), c2, eps, lam, inv_norm, wtab,
-                                                           wtab_panels);
+    k_spectrum_finalize<double><<<blocks_for(total), threads, 0, s>>>(O, (double*)out, (int)kernel, n0, n1, n2, cs[0],
+                                                                      cs[1], c2, eps, lam, inv_norm, wtab, wtab_panels);
   else
-    k_spectrum_finalize<float><<<blocks, threads, 0, s>>>(O, (float*)out, (int)kernel, n0, n1, n2, pi / (2 * L[0]),
-                                                          pi / (2 * L[1]), c2, eps, lam, inv_norm, wtab,
-                                                          wtab_panels);
+    k_spectrum_finalize<float><<<blocks_for(total), threads, 0, s>>>(O, (float*)out, (int)kernel, n0, n1, n2, cs[0],
+                                                                     cs[1], c2, eps, lam, inv_norm, wtab, wtab_panels);
   return cudaGetLastError();
 }
 
