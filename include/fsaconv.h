@@ -379,9 +379,9 @@ fsa_status fsa_profiler_destroy(fsa_profiler* prof);
  * each thread holds half the values and twice the warps fit on an SM
  * (lengths 128, 192, 256, 384, 512; generation 4's middle pass elsewhere);
  * generation 8 = generation 4 with a middle pass and the axis-0 R2C and C2R
- * passes whose column tiles are staged by tiled bulk tensor copies (TMA),
- * bit-equal to generation 2's (same lengths; one tensor map per solve of a
- * launch).
+ * passes whose column tiles are staged by tiled bulk tensor copies (TMA;
+ * lengths 128 to 1024, one tensor map per solve of a launch): bit-equal to
+ * generation 2's, the middle pass of lengths 768 and 1024 within round-off.
  * mode 1 (default): each new FP32 plan times every generation for
  * each of its passes on its own workspace at creation and keeps the fastest
  * per (pass, length); choices persist for the process.  mode 0: untuned

@@ -60,6 +60,15 @@ template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
 template <typename V> __device__ __forceinline__ V cmulc(V a, V b) {
   return mk(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
+// FP32: the fused form written out, so that every kernel rounds alike whatever
+// the twiddle was loaded from (left to the compiler, the product it fuses
+// depends on that).
+template <> __device__ __forceinline__ float2 cmul<float2>(float2 a, float2 b) {
+  return mk(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+template <> __device__ __forceinline__ float2 cmulc<float2>(float2 a, float2 b) {
+  return mk(__fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, -__fmul_rn(a.x, b.y)));
+}
 template <typename V> __device__ __forceinline__ V cscale(V a, typename RealOf<V>::T s) { return mk(a.x * s, a.y * s); }
 
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000

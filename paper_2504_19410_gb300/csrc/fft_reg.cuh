@@ -48,7 +48,11 @@ template <int R, int E, bool FWD, typename V> __device__ __forceinline__ V twc(V
     constexpr int k = e * (96 / R);
     constexpr T c = (T)Tw96::c[k];
     constexpr T s = FWD ? (T)(-Tw96::s[k]) : (T)Tw96::s[k];
-    return mk(a.x * c - a.y * s, a.x * s + a.y * c);
+    // FP32: fused as in cmul (fft_core.cuh), whatever kernel it is part of
+    if constexpr (std::is_same<T, float>::value)
+      return mk(__fmaf_rn(a.x, c, -__fmul_rn(a.y, s)), __fmaf_rn(a.x, s, __fmul_rn(a.y, c)));
+    else
+      return mk(a.x * c - a.y * s, a.x * s + a.y * c);
   }
 }
 
@@ -153,12 +157,26 @@ template <> struct Plan2For<512> { using type = Plan2<512, 16, 32>; };
 template <> struct Plan2For<768> { using type = Plan2<768, 24, 32>; };
 template <> struct Plan2For<1024> { using type = Plan2<1024, 32, 32>; };
 
+// Twiddle sources of the steps: tw(e) = exp(-2 pi i e / M), 0 <= e < M, from
+// the unit's table in HBM, or from a copy of the length's M values in shared
+// memory (TwShared, filled by tw_copy).
+template <int M, typename V> struct TwGlobal {
+  __device__ __forceinline__ V operator()(int e) const { return twiddle<V, M>(e); }
+};
+struct TwShared {
+  const float2* w;
+  __device__ __forceinline__ float2 operator()(int e) const { return w[e]; }
+};
+template <int M> __device__ __forceinline__ void tw_copy(float2* w) {
+  for (int e = threadIdx.x; e < M; e += blockDim.x) w[e] = twiddle<float2, M>(e);
+}
+
 // Step A, forward: thread u handles t = u, u + T, ... < R2.  ld(t, r) returns
 // x[t + R2 r]; st(q, t, v) stores the twiddled result for (q, t).
 // With HALF (the pruned passes: x[t + R2 r] = 0 for r >= R1/2), only the
 // lower half is loaded and the half-input transform is used (R1 even).
-template <class P, typename V, bool HALF = false, class Ld, class St>
-__device__ __forceinline__ void stepA_fwd(int u, const Ld& ld, const St& st) {
+template <class P, typename V, bool HALF = false, class Ld, class St, class Tw = TwGlobal<P::M, V>>
+__device__ __forceinline__ void stepA_fwd(int u, const Ld& ld, const St& st, const Tw& tw = Tw()) {
   constexpr int R1 = P::R1, R2 = P::R2;
   constexpr bool H = HALF && (R1 % 2 == 0);
 #pragma unroll
@@ -176,7 +194,7 @@ __device__ __forceinline__ void stepA_fwd(int u, const Ld& ld, const St& st) {
         rfft<R1, true>(a);
       }
 #pragma unroll
-      for (int q = 1; q < R1; ++q) a[q] = cmul(a[q], twiddle<V, P::M>(t * q));
+      for (int q = 1; q < R1; ++q) a[q] = cmul(a[q], tw(t * q));
 #pragma unroll
       for (int q = 0; q < R1; ++q) st(q, t, a[q]);
     }
@@ -212,11 +230,11 @@ __device__ __forceinline__ void stepA_inv(int u, const Ld& ld, const St& st) {
 
 // Step B, inverse tail: b[s] (s < R2) of sub-transform q -> inverse length-R2
 // transform -> multiplied by exp(+2 pi i t q / M) -> st(q, t, v).
-template <class P, typename V, class St>
-__device__ __forceinline__ void stepB_inv(int q, V* b, const St& st) {
+template <class P, typename V, class St, class Tw = TwGlobal<P::M, V>>
+__device__ __forceinline__ void stepB_inv(int q, V* b, const St& st, const Tw& tw = Tw()) {
   rfft<P::R2, false>(b);
 #pragma unroll
-  for (int t = 0; t < P::R2; ++t) st(q, t, t == 0 ? b[0] : cmulc(b[t], twiddle<V, P::M>(t * q)));
+  for (int t = 0; t < P::R2; ++t) st(q, t, t == 0 ? b[0] : cmulc(b[t], tw(t * q)));
 }
 
 }  // namespace fsa

@@ -1,5 +1,5 @@
 // FP32 eighth-generation middle, R2C and C2R passes (passes8.cuh): the column
-// tiles staged by tiled bulk tensor copies, lengths 128 to 512.  Compiled as
+// tiles staged by tiled bulk tensor copies, lengths 128 to 1024.  Compiled as
 // its own translation unit; the launchers are looked up by length (k8_colm,
 // k8_colm_shared, k8_r2c, k8_c2r) when the other FP32 instances register
 // their function tables.  A launch whose buffers a tensor map cannot describe
@@ -49,17 +49,22 @@ bool encode_2d(CUtensorMap* map, const void* base, CUtensorMapDataType dt, int e
 
 template <int M> struct Inst8 {
   using P = typename Plan2For<M>::type;
-  using G = Geo8<P>;
+  static constexpr bool WIDE = M > 512;  // the long lines' middle pass
+  using G = typename std::conditional<WIDE, Geo8W<P>, Geo8<P>>::type;
   using GR = Geo8R<P>;
   using GC = Geo8C<P>;
+  template <int NJ, bool SHARED> static constexpr auto mid_kernel() {
+    if constexpr (WIDE) return k8w_col_mid<P, NJ, SHARED>;
+    else return k8_col_mid<P, NJ, SHARED>;
+  }
   static cudaError_t prepare() {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void* f, int bytes) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-    set((const void*)k8_col_mid<P, 1>, G::SMEM);
-    set((const void*)k8_col_mid<P, kMaxJobs>, G::SMEM);
-    set((const void*)k8_col_mid<P, kMaxJobs, true>, G::SMEM);
+    set((const void*)mid_kernel<1, false>(), G::SMEM);
+    set((const void*)mid_kernel<kMaxJobs, false>(), G::SMEM);
+    set((const void*)mid_kernel<kMaxJobs, true>(), G::SMEM);
     set((const void*)k8_r2c_ax0<P, 1>, GR::SMEM);
     set((const void*)k8_r2c_ax0<P, kMaxJobs>, GR::SMEM);
     set((const void*)k8_c2r_ax0<P, 1>, GC::SMEM);
@@ -67,11 +72,17 @@ template <int M> struct Inst8 {
     return e;
   }
   // The C2R pass: X of each solve as a {C, n0 + 1} tensor of 8-byte elements.
+  // The long lines read 64-byte rows; where those lie more than 1.5 MB apart
+  // (each then costs a page translation of its own) generation 2's 256-byte
+  // rows are faster: length 1024 at C = 512^2, 0.434 against 0.488 ms (at C =
+  // 512 x 128 0.116 against 0.079, length 768 at C = 384^2 0.195 against 0.177).
+  static constexpr long long kFarRows = 200000;
   template <int NJ> static cudaError_t c2r_n(const Jobs& jobs, long long C, cudaStream_t s) {
+    if (WIDE && C > kFarRows) return pass_fns(kArithF32G2, M).c2r(jobs, C, s);
     TmapSet<NJ> maps;
     for (int j = 0; j < jobs.count; ++j)
       if (!encode_2d(&maps.m[j], jobs.j[j].in, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, C, M / 2 + 1, 2 * GC::W,
-                     GC::ROWS / 2))
+                     GC::BOX))
         return pass_fns(kArithF32G2, M).c2r(jobs, C, s);
     Jobs jj = jobs;
     jj.fault = device_fault_word();
@@ -90,7 +101,7 @@ template <int M> struct Inst8 {
   template <int NJ> static cudaError_t r2c_n(const Jobs& jobs, long long C, cudaStream_t s) {
     TmapSet<NJ> maps;
     for (int j = 0; j < jobs.count; ++j)
-      if (!encode_2d(&maps.m[j], jobs.j[j].in, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, C, M / 2, 2 * GR::W, M / 2))
+      if (!encode_2d(&maps.m[j], jobs.j[j].in, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, C, M / 2, 2 * GR::W, GR::BOXROWS))
         return pass_fns(kArithF32G2, M).r2c(jobs, C, s);
     Jobs jj = jobs;
     jj.fault = device_fault_word();
@@ -106,19 +117,22 @@ template <int M> struct Inst8 {
   // 8-byte elements; the same fallback.
   template <int NJ, bool SHARED = false>
   static cudaError_t colm_n(const Jobs& jobs, int M2, int planes, cudaStream_t s) {
-    constexpr int n1 = M / 2;
+    constexpr int n1 = M / 2, boxrows = n1 > 256 ? n1 / 2 : n1;
     TmapSet<NJ> maps;
     for (int j = 0; j < jobs.count; ++j)
       if (M2 % G::W != 0 || !encode_2d(&maps.m[j], jobs.j[j].out, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, M2,
-                                       (long long)planes * n1, G::W, n1))
+                                       (long long)planes * n1, G::W, boxrows))
         return SHARED ? pass_fns(kArithF32G3, M).colm_shared(jobs, M2, planes, s)
                       : pass_fns(kArithF32G2, M).colm(jobs, M2, planes, s);
     Jobs jj = jobs;
     jj.fault = device_fault_word();
-    // SHARED: one CTA slot per tile (each walks the tile for every solve)
+    // SHARED: one CTA slot per tile (each walks the tile for every solve); the
+    // long lines' kernel takes one CTA per tile and hands the tiles out itself
     const long long tiles = (long long)(M2 / G::W) * planes * (SHARED ? 1 : jobs.count);
-    auto f = k8_col_mid<P, NJ, SHARED>;
-    f<<<persistent_grid((const void*)f, G::NT, G::SMEM, tiles), G::NT, G::SMEM, s>>>(jj, M2, planes, maps);
+    if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
+    const auto f = mid_kernel<NJ, SHARED>();
+    const int grid = WIDE ? (int)tiles : persistent_grid((const void*)f, G::NT, G::SMEM, tiles);
+    f<<<grid, G::NT, G::SMEM, s>>>(jj, M2, planes, maps);
     return cudaGetLastError();
   }
   static cudaError_t colm(const Jobs& jobs, int M2, int planes, cudaStream_t s) {
@@ -139,6 +153,8 @@ ColmFn k8_colm_shared(int M) {
     case 256: return &Inst8<256>::colm_shared;
     case 384: return &Inst8<384>::colm_shared;
     case 512: return &Inst8<512>::colm_shared;
+    case 768: return &Inst8<768>::colm_shared;
+    case 1024: return &Inst8<1024>::colm_shared;
     default: return nullptr;
   }
 }
@@ -150,6 +166,8 @@ ColmFn k8_colm(int M) {
     case 256: return &Inst8<256>::colm;
     case 384: return &Inst8<384>::colm;
     case 512: return &Inst8<512>::colm;
+    case 768: return &Inst8<768>::colm;
+    case 1024: return &Inst8<1024>::colm;
     default: return nullptr;
   }
 }
@@ -161,6 +179,8 @@ R2cFn k8_r2c(int M) {
     case 256: return &Inst8<256>::r2c;
     case 384: return &Inst8<384>::r2c;
     case 512: return &Inst8<512>::r2c;
+    case 768: return &Inst8<768>::r2c;
+    case 1024: return &Inst8<1024>::r2c;
     default: return nullptr;
   }
 }
@@ -172,6 +192,8 @@ R2cFn k8_c2r(int M) {
     case 256: return &Inst8<256>::c2r;
     case 384: return &Inst8<384>::c2r;
     case 512: return &Inst8<512>::c2r;
+    case 768: return &Inst8<768>::c2r;
+    case 1024: return &Inst8<1024>::c2r;
     default: return nullptr;
   }
 }
@@ -183,6 +205,8 @@ cudaError_t k8_prepare(int M) {
     case 256: return Inst8<256>::prepare();
     case 384: return Inst8<384>::prepare();
     case 512: return Inst8<512>::prepare();
+    case 768: return Inst8<768>::prepare();
+    case 1024: return Inst8<1024>::prepare();
     default: return cudaSuccess;
   }
 }

@@ -46,7 +46,7 @@
 // q (k_radial_tables) and looked up by the first and the last DCT pass, which
 // saves their per-point evaluation on the FP64 pipe and three passes over
 // the octant.  Measured (GB300, FP64 plan of 256^3): octant
-// 2.60 and spectrum 0.89 ms before, 0.05 ms for the tables now; with the
+// 2.60 and spectrum 0.89 ms before, 0.11 ms for the tables now; with the
 // pruned DCT passes the whole generation 6.65 -> 2.00 ms.
 // Other grids (no common integer ratio, or a table above a quarter of the
 // octant: planes, very flat boxes) evaluate per point.
