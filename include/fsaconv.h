@@ -384,7 +384,8 @@ fsa_status fsa_profiler_destroy(fsa_profiler* prof);
  * generation 2's, the middle pass of lengths 768 and 1024 within round-off.
  * mode 1 (default): each new FP32 plan times every generation for
  * each of its passes on its own workspace at creation and keeps the fastest
- * per (pass, length); choices persist for the process.  mode 0: untuned
+ * per (pass, length, whether the solve's intermediates fit in L2); choices
+ * persist for the process.  mode 0: untuned
  * passes use generation 2.  mode 2 / 3 / 4 / 5 / 6 / 7: force generation
  * 1 / 2 / 3 / 4 / 6 / 8 for every FP32 pass.  FP64 plans compute either in native FP64 or in
  * double-word arithmetic (two floats, 48-bit significand, on the FP32 pipes;

@@ -32,10 +32,17 @@ struct Geometry {
 
 bool supported_n(int n);
 int& autotune_mode();  // fsa_autotune_set: 0 defaults, 1 tune per plan, 2..5 force generation 1..4
-// Kernel generation used for a pass of length M in a dtype: 1 = Stockham
-// radix-8 (passes.cuh), 2 = two-step register kernels (passes2.cuh, FP32).
-int kernel_variant(int pass, int M, fsa_dtype dt);
-void set_kernel_variant(int pass, int M, fsa_dtype dt, int variant);
+// Size class of an FP32 grid: 0 where its X and Y (24 bytes a point) stay in
+// the 129 MB L2 from pass to pass, 1 where they stream through HBM.  The tuner
+// chooses per class: the kernel that wins on a resident 96 x 48 x 192 solve
+// (row inverse, length 384) took 62 instead of 56 us at 192^3, one picked at
+// 128^3 (row forward, length 256) 235 instead of 178 us at 512 x 512 x 128.
+constexpr long long kCachedBytes = 96LL << 20;
+int size_class(const int* n);
+// Kernel generation used for an FP32 pass of length M (variant numbers as
+// arith_of_variant in plan.cu).
+int kernel_variant(int pass, int M, int cls);
+void set_kernel_variant(int pass, int M, int cls, int variant);
 bool supported_M(int M);
 
 // Launchers of one kernel instance (one arithmetic, one transform length M),
@@ -144,10 +151,10 @@ int mixed_launches(int count, bool pipelined);  // launches mixed_passes makes f
 int& batched_mode();
 // The fused outer pass pair used for FP32 grids with n0 = n2 and transform
 // length M = 2 n0 (dir 0 forward, 1 inverse): 0 = the separate passes, c >= 1
-// = fused cluster configuration c - 1.  set_fused_config(M, dir, -1) leaves
+// = fused cluster configuration c - 1.  set_fused_config(M, dir, cls, -1) leaves
 // the choice to the tuner.
-int fused_config(int M, int dir);
-void set_fused_config(int M, int dir, int c);
+int fused_config(int M, int dir, int cls);
+void set_fused_config(int M, int dir, int cls, int c);
 // This device's fault word (Jobs::fault), allocated by prepare_device;
 // ensure_device_fault_word allocates it if needed (current device).
 unsigned int* device_fault_word();

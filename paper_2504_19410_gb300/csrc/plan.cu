@@ -104,32 +104,35 @@ int& autotune_mode() {
 }
 
 namespace {
-// Chosen generation per (pass, transform length, dtype); 0 = not chosen yet.
+// Chosen generation per (pass, transform length, size class) of the FP32
+// passes; 0 = not chosen yet.
 std::atomic<signed char> g_variant[kNumPass][1025][2];
 std::mutex g_tune_mu;
 }  // namespace
 
-int kernel_variant(int pass, int M, fsa_dtype dt) {
+int size_class(const int* n) { return (long long)(n[0] + 1) * n[1] * n[2] * 24 > kCachedBytes ? 1 : 0; }
+
+int kernel_variant(int pass, int M, int cls) {
   const int mode = autotune_mode();
-  if (dt == FSA_F64) return 1;
   if (mode == 2) return 1;
   if (mode == 3) return 2;
   if (mode == 4) return 3;
   if (mode == 5) return 4;
   if (mode == 6) return pass == kColMid ? 5 : 4;
   if (mode == 7) return 6;  // generation 8's table: generation 4 elsewhere
-  const int v = (M >= 0 && M <= 1024) ? g_variant[pass][M][dt].load(std::memory_order_relaxed) : 0;
+  const int v = (M >= 0 && M <= 1024) ? g_variant[pass][M][cls].load(std::memory_order_relaxed) : 0;
   return v ? v : 2;
 }
 
-void set_kernel_variant(int pass, int M, fsa_dtype dt, int variant) {
-  if (M >= 0 && M <= 1024) g_variant[pass][M][dt].store((signed char)variant, std::memory_order_relaxed);
+void set_kernel_variant(int pass, int M, int cls, int variant) {
+  if (M >= 0 && M <= 1024) g_variant[pass][M][cls].store((signed char)variant, std::memory_order_relaxed);
 }
 
 namespace {
-// Fused outer pair per (length, direction): -1 unpinned and untuned, else as
-// fused_config.  Pins (fsa_fused_select) and tuner results share the table.
-std::atomic<signed char> g_fused[1025][2];
+// Fused outer pair per (length, direction, size class): -1 unpinned and
+// untuned, else as fused_config.  Pins (fsa_fused_select) and tuner results
+// share the table.
+std::atomic<signed char> g_fused[1025][2][2];
 std::atomic<bool> g_fused_init{false};
 void fused_table_init() {
   if (g_fused_init.load()) return;
@@ -137,25 +140,26 @@ void fused_table_init() {
   std::lock_guard<std::mutex> lk(mu);
   if (g_fused_init.load()) return;
   for (auto& m : g_fused)
-    for (auto& d : m) d.store(-1);
+    for (auto& d : m)
+      for (auto& c : d) c.store(-1);
   g_fused_init.store(true);
 }
 }  // namespace
 
-int fused_config(int M, int dir) {
+int fused_config(int M, int dir, int cls) {
   const int mode = autotune_mode();
   if (mode >= 2 || M < 0 || M > 1024 || dir < 0 || dir > 1) return 0;
   const int nf = pass_fns(kArithF32G5, M).nfused;
   if (nf == 0) return 0;
   fused_table_init();
-  const int c = g_fused[M][dir].load(std::memory_order_relaxed);
+  const int c = g_fused[M][dir][cls].load(std::memory_order_relaxed);
   return c >= 0 && c <= nf ? c : 0;  // unpinned and untuned: the separate passes
 }
 
-void set_fused_config(int M, int dir, int c) {
+void set_fused_config(int M, int dir, int cls, int c) {
   if (M < 0 || M > 1024 || dir < 0 || dir > 1) return;
   fused_table_init();
-  g_fused[M][dir].store((signed char)c, std::memory_order_relaxed);
+  g_fused[M][dir][cls].store((signed char)c, std::memory_order_relaxed);
 }
 
 namespace {
@@ -241,9 +245,9 @@ int arith_of_variant(int v) {
                   : (v == 3 ? kArithF32G3 : (v == 2 ? kArithF32G2 : kArithF32G1));
 }
 
-template <typename V> int arith_for(int pass, int M) {
+template <typename V> int arith_for(int pass, int M, int cls) {
   if constexpr (std::is_same<V, float2>::value) {
-    return arith_of_variant(kernel_variant(pass, M, FSA_F32));
+    return arith_of_variant(kernel_variant(pass, M, cls));
   }
   else if constexpr (std::is_same<V, double2>::value)
     return kArithF64;
@@ -293,7 +297,7 @@ template <typename V> int fused_pair(const int* n, int dir) {
     return 0;
   } else {
     if (n[0] != n[2]) return 0;
-    return fused_config(2 * n[0], dir);
+    return fused_config(2 * n[0], dir, size_class(n));
   }
 }
 
@@ -304,6 +308,7 @@ cudaError_t group_passes(const int* n, int count, const void* const* rho, void* 
   const int n0 = n[0], n1 = n[1], n2 = n[2];
   const long long C = (long long)n1 * n2;
   const long long rows = (long long)(n0 + 1) * n1;
+  const int cls = size_class(n);
   cudaError_t e = cudaSuccess;
   for (int b = 0; b < count && e == cudaSuccess; b += kMaxJobs) {
     const int m = count - b < kMaxJobs ? count - b : kMaxJobs;
@@ -318,11 +323,11 @@ cudaError_t group_passes(const int* n, int count, const void* const* rho, void* 
       j5.j[i] = Job{X[k], phi[k], nullptr};
     }
     if (e == cudaSuccess) e = trace_mark(tr, -1, s);
-    const PassFns& f1 = pass_fns(arith_for<V>(kR2C, 2 * n0), 2 * n0);
-    const PassFns& f2 = pass_fns(arith_for<V>(kRowFwd, 2 * n2), 2 * n2);
-    const PassFns& f3 = pass_fns(arith_for<V>(kColMid, 2 * n1), 2 * n1);
-    const PassFns& f4 = pass_fns(arith_for<V>(kRowInv, 2 * n2), 2 * n2);
-    const PassFns& f5 = pass_fns(arith_for<V>(kC2R, 2 * n0), 2 * n0);
+    const PassFns& f1 = pass_fns(arith_for<V>(kR2C, 2 * n0, cls), 2 * n0);
+    const PassFns& f2 = pass_fns(arith_for<V>(kRowFwd, 2 * n2, cls), 2 * n2);
+    const PassFns& f3 = pass_fns(arith_for<V>(kColMid, 2 * n1, cls), 2 * n1);
+    const PassFns& f4 = pass_fns(arith_for<V>(kRowInv, 2 * n2, cls), 2 * n2);
+    const PassFns& f5 = pass_fns(arith_for<V>(kC2R, 2 * n0, cls), 2 * n0);
     if (!f1.r2c || !f2.rowf || !f3.colm || !f4.rowi || !f5.c2r) return cudaErrorInvalidValue;
     // pass split: slabs of planes whose X + Y fit chunk_bytes stay in L2
     // between the row-forward, middle and row-inverse passes
@@ -457,12 +462,13 @@ cudaError_t group_passes_ddi(const fsa_plan* shape, int count, const void* const
   const long long C = (long long)n1 * n2;
   const long long rows = (long long)(n0 + 1) * n1;
   const bool grid = shape->ddi == FSA_DDI_GRID;
+  const int cls = size_class(shape->n);
   if (!par) return cudaErrorInvalidValue;
-  const PassFns& f1 = pass_fns(arith_for<V>(kR2C, 2 * n0), 2 * n0);
-  const PassFns& f2 = pass_fns(arith_for<V>(kRowFwd, 2 * n2), 2 * n2);
-  const PassFns& f3 = pass_fns(arith_for<V>(kColMid, 2 * n1), 2 * n1);
-  const PassFns& f4 = pass_fns(arith_for<V>(kRowInv, 2 * n2), 2 * n2);
-  const PassFns& f5 = pass_fns(arith_for<V>(kC2R, 2 * n0), 2 * n0);
+  const PassFns& f1 = pass_fns(arith_for<V>(kR2C, 2 * n0, cls), 2 * n0);
+  const PassFns& f2 = pass_fns(arith_for<V>(kRowFwd, 2 * n2, cls), 2 * n2);
+  const PassFns& f3 = pass_fns(arith_for<V>(kColMid, 2 * n1, cls), 2 * n1);
+  const PassFns& f4 = pass_fns(arith_for<V>(kRowInv, 2 * n2, cls), 2 * n2);
+  const PassFns& f5 = pass_fns(arith_for<V>(kC2R, 2 * n0, cls), 2 * n0);
   if (!f1.r2c || !f2.rowf || !f3.colm || !f3.colm_ddi || !f4.rowi || !f5.c2r || !f5.c2r_epi)
     return cudaErrorInvalidValue;
   // unpadded passes: the bulk-copy generation for FP32, first generation in
@@ -783,7 +789,8 @@ fsa_status fsa_fused_select(int M, int dir, int c) {
   if (dir < 0 || dir > 2) return set_error(FSA_ERR_INVALID_ARG, "fsa_fused_select: dir must be 0, 1 or 2");
   if (c < -1 || c > nf) return set_error(FSA_ERR_INVALID_ARG, "fsa_fused_select: configuration out of range");
   for (int d = 0; d < 2; ++d)
-    if (dir == 2 || dir == d) set_fused_config(M, d, c);
+    if (dir == 2 || dir == d)
+      for (int cls = 0; cls < 2; ++cls) set_fused_config(M, d, cls, c);
   apply_graphs_invalidate();
   return FSA_OK;
 }
@@ -1013,7 +1020,7 @@ size_t ddi_table(const fsa_plan* p, const DdiPar& b, void* out) {
 
 // Autotuner: for an FP32 plan, time both kernel generations of each pass on the
 // plan's own workspace (contents irrelevant: the kernels' cost does not depend
-// on the data) and keep the faster for that pass and length.
+// on the data) and keep the faster for that pass, length and size class.
 cudaError_t tune_f64(fsa_plan* p);
 
 cudaError_t tune_plan(fsa_plan* p) {
@@ -1022,12 +1029,13 @@ cudaError_t tune_plan(fsa_plan* p) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   const int n0 = p->n[0], n1 = p->n[1], n2 = p->n[2];
   const int Ms[kNumPass] = {2 * n0, 2 * n2, 2 * n1, 2 * n2, 2 * n0};
+  const int cls = size_class(p->n);
   bool need = false;
-  for (int k = 0; k < kNumPass; ++k) need |= g_variant[k][Ms[k]][FSA_F32].load() == 0;
+  for (int k = 0; k < kNumPass; ++k) need |= g_variant[k][Ms[k]][cls].load() == 0;
   const PassFns& f5g = pass_fns(kArithF32G5, 2 * n0);
   fused_table_init();
   const bool fuse = n0 == n2 && f5g.nfused > 0;
-  for (int dir = 0; dir < 2 && fuse; ++dir) need |= g_fused[2 * n0][dir].load() < 0;
+  for (int dir = 0; dir < 2 && fuse; ++dir) need |= g_fused[2 * n0][dir][cls].load() < 0;
   if (!need) return cudaSuccess;
   cudaStream_t s;
   cudaEvent_t e0, e1;
@@ -1055,7 +1063,7 @@ cudaError_t tune_plan(fsa_plan* p) {
   for (int rep = 0; rep < 20 && e == cudaSuccess; ++rep) e = run(kColMid, 2);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   for (int k = 0; k < kNumPass && e == cudaSuccess; ++k) {
-    if (g_variant[k][Ms[k]][FSA_F32].load() != 0) continue;
+    if (g_variant[k][Ms[k]][cls].load() != 0) continue;
     // variants 5 and 6 (the sixth-generation middle pass, the
     // eighth-generation middle, R2C and C2R passes) only where they exist
     std::vector<int> cand = {1, 2, 3, 4};
@@ -1084,21 +1092,21 @@ cudaError_t tune_plan(fsa_plan* p) {
     int pick = 2;
     for (int v : cand)
       if (tmin[v] < tmin[pick]) pick = v;
-    set_kernel_variant(k, Ms[k], FSA_F32, e == cudaSuccess ? pick : 0);
+    set_kernel_variant(k, Ms[k], cls, e == cudaSuccess ? pick : 0);
   }
   // the fused outer pairs against the separate passes just chosen (X stands
   // in for rho and phi: the kernels' cost does not depend on the data)
   auto run_pair = [&](int dir, int c) -> cudaError_t {
     if (c == 0) {
       const int a = dir == 0 ? kR2C : kRowInv, b = dir == 0 ? kRowFwd : kC2R;
-      cudaError_t r = run(a, kernel_variant(a, Ms[a], FSA_F32));
-      return r == cudaSuccess ? run(b, kernel_variant(b, Ms[b], FSA_F32)) : r;
+      cudaError_t r = run(a, kernel_variant(a, Ms[a], cls));
+      return r == cudaSuccess ? run(b, kernel_variant(b, Ms[b], cls)) : r;
     }
     j.j[0] = dir == 0 ? Job{X, Y, nullptr} : Job{Y, X, nullptr};
     return dir == 0 ? f5g.fwd5(c - 1, j, n1, s) : f5g.inv5(c - 1, j, n1, s);
   };
   for (int dir = 0; dir < 2 && fuse && e == cudaSuccess; ++dir) {
-    if (g_fused[2 * n0][dir].load() >= 0) continue;
+    if (g_fused[2 * n0][dir][cls].load() >= 0) continue;
     float best = 1e30f;
     int pick = 0;
     for (int c = 0; c <= f5g.nfused && e == cudaSuccess; ++c) {
@@ -1124,7 +1132,7 @@ cudaError_t tune_plan(fsa_plan* p) {
         pick = c;
       }
     }
-    if (e == cudaSuccess) set_fused_config(2 * n0, dir, pick);
+    if (e == cudaSuccess) set_fused_config(2 * n0, dir, cls, pick);
   }
   cudaStreamSynchronize(s);
   cudaEventDestroy(e0);
