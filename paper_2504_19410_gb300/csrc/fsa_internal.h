@@ -69,6 +69,8 @@ struct PassFns {
   // the middle pass for jobs that all share one spectrum (densities of one
   // plan): one spectrum read per column tile where the generation has it
   cudaError_t (*colm_shared)(const Jobs&, int M2, int planes, cudaStream_t) = nullptr;
+  // its prefetching (cp.async) form, for buffers a tensor map cannot describe (generation 3's table)
+  cudaError_t (*colm_shared_p)(const Jobs&, int M2, int planes, cudaStream_t) = nullptr;
   cudaError_t (*c2r_epi)(const Jobs&, long long C, cudaStream_t) = nullptr;
   cudaError_t (*r2c_per)(const Jobs&, long long C, cudaStream_t) = nullptr;
   cudaError_t (*rowf_per)(const Jobs&, long long rows, cudaStream_t) = nullptr;
@@ -109,7 +111,8 @@ cudaError_t k6_prepare(int M);
 // The eighth-generation middle pass (passes8.cuh, inst_f32g8.cu): column tiles
 // staged by one tiled bulk tensor copy each; null where it has no instance.
 ColmFn k8_colm(int M);
-ColmFn k8_colm_shared(int M);  // its form for densities of one plan (one spectrum read per tile)
+ColmFn k8_colm_shared(int M);  // its form for densities of one plan (one spectrum read per run)
+ColmFn k8_colm_shared_exact(int M);  // the same where it is bit-equal to generation 2 (M <= 512)
 using R2cFn = cudaError_t (*)(const Jobs&, long long, cudaStream_t);
 R2cFn k8_r2c(int M);  // the R2C pass staged the same way
 R2cFn k8_c2r(int M);  // and the C2R pass (same launcher signature)
@@ -166,6 +169,13 @@ cudaError_t init_all_twiddles();  // every instance unit's tables, current devic
 
 // Resident CTAs per SM for a kernel (cached per function), times the SM count.
 int persistent_grid(const void* func, int threads, int smem, long long tiles);
+// How many solves of one column tile a CTA of the shared-spectrum middle pass
+// takes in a row (it reads the tile's spectrum values once per run): the
+// largest divisor of `count` whose runs fill at least nine tenths of the
+// resident CTAs' rounds.  With all solves of a tile in one run, 64 densities
+// of 64^3 were 520 runs for 456 CTAs, two rounds; shorter runs read the
+// spectrum again, from L2.
+int shared_run(const void* func, int threads, int smem, long long tiles, int count);
 // Grid policy of the calling host thread's launches: 0 = persistent grids
 // (resident CTAs x SMs, the default), 1 = one CTA per tile, so that the
 // blocks of a long solve retire one tile at a time and kernels of

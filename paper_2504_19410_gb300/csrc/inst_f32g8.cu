@@ -122,17 +122,24 @@ template <int M> struct Inst8 {
     for (int j = 0; j < jobs.count; ++j)
       if (M2 % G::W != 0 || !encode_2d(&maps.m[j], jobs.j[j].out, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, M2,
                                        (long long)planes * n1, G::W, boxrows))
-        return SHARED ? pass_fns(kArithF32G3, M).colm_shared(jobs, M2, planes, s)
+        return SHARED ? pass_fns(kArithF32G3, M).colm_shared_p(jobs, M2, planes, s)
                       : pass_fns(kArithF32G2, M).colm(jobs, M2, planes, s);
     Jobs jj = jobs;
     jj.fault = device_fault_word();
-    // SHARED: one CTA slot per tile (each walks the tile for every solve); the
-    // long lines' kernel takes one CTA per tile and hands the tiles out itself
-    const long long tiles = (long long)(M2 / G::W) * planes * (SHARED ? 1 : jobs.count);
-    if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
+    // SHARED: runs of several solves of one tile; the long lines' kernel takes
+    // one CTA per tile (SHARED: of one solve) and hands the tiles out itself
+    const long long tpj = (long long)(M2 / G::W) * planes;
     const auto f = mid_kernel<NJ, SHARED>();
-    const int grid = WIDE ? (int)tiles : persistent_grid((const void*)f, G::NT, G::SMEM, tiles);
-    f<<<grid, G::NT, G::SMEM, s>>>(jj, M2, planes, maps);
+    int run = 1, grid = 0;
+    if constexpr (WIDE) {
+      const long long tiles = SHARED ? tpj : tpj * jobs.count;
+      if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
+      grid = (int)tiles;
+    } else {
+      if (SHARED) run = shared_run((const void*)f, G::NT, G::SMEM, tpj, jobs.count);
+      grid = persistent_grid((const void*)f, G::NT, G::SMEM, tpj * jobs.count / run);
+    }
+    f<<<grid, G::NT, G::SMEM, s>>>(jj, M2, planes, run, maps);
     return cudaGetLastError();
   }
   static cudaError_t colm(const Jobs& jobs, int M2, int planes, cudaStream_t s) {
@@ -158,6 +165,8 @@ ColmFn k8_colm_shared(int M) {
     default: return nullptr;
   }
 }
+
+ColmFn k8_colm_shared_exact(int M) { return M <= 512 ? k8_colm_shared(M) : nullptr; }
 
 ColmFn k8_colm(int M) {
   switch (M) {

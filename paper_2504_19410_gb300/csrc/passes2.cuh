@@ -278,10 +278,11 @@ template <class P> struct Stage2 {
 };
 
 // SHARED: every job of the launch has the same spectrum (densities of one
-// plan).  A CTA then takes a column tile for all jobs in turn and loads the
-// tile's spectrum values once (one spectrum read per tile, not per job).
+// plan).  A CTA then takes a column tile for `run` jobs in turn and loads the
+// tile's spectrum values once per run (run divides the job count: shared_run).
 template <class P, int MODE = kMulSpectrum, bool SHARED = false>
-__global__ void __launch_bounds__(Geo2<P>::NT, Geo2<P>::MINB_MID) k2p_col_mid(const Jobs jobs, int M2, int planes) {
+__global__ void __launch_bounds__(Geo2<P>::NT, Geo2<P>::MINB_MID) k2p_col_mid(const Jobs jobs, int M2, int planes,
+                                                                                          int run = 1) {
   using V = float2;
   constexpr int M = P::M, n = M / 2, W = Geo2<P>::W, R1 = P::R1, R2 = P::R2, T = P::T;
   constexpr int RA = Stage2<P>::RA;
@@ -300,10 +301,10 @@ __global__ void __launch_bounds__(Geo2<P>::NT, Geo2<P>::MINB_MID) k2p_col_mid(co
   auto job_of = [&](long long tile) -> int { return (int)(SHARED ? ph(tile) % K : ph(tile) / tpj); };
   auto lt_of = [&](long long tile) -> int { return (int)(SHARED ? ph(tile) / K : ph(tile) % tpj); };
   auto next_of = [&](long long tile) -> long long {
-    if constexpr (SHARED) return tile % K + 1 < K ? tile + 1 : (tile / K + gridDim.x) * K;
+    if constexpr (SHARED) return tile % run + 1 < run ? tile + 1 : (tile / run + gridDim.x) * run;
     else return tile + gridDim.x;
   };
-  const long long first = SHARED ? (long long)blockIdx.x * K : (long long)blockIdx.x;
+  const long long first = SHARED ? (long long)blockIdx.x * run : (long long)blockIdx.x;
   auto issue = [&](long long tile) {
     const Job& jb = jobs.j[job_of(tile)];
     const int lt = lt_of(tile);
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(Geo2<P>::NT, Geo2<P>::MINB_MID) k2p_col_mid(co
     if (next_of(tile) < total) issue(next_of(tile));
     __syncthreads();
     // SHARED: the first job of the group this CTA takes in turn loads the tile's spectrum
-    if (!SHARED || tile % K == 0) mid_load<P>(sp, srow, u, ok, n2 + 1);
+    if (!SHARED || tile % run == 0) mid_load<P>(sp, srow, u, ok, n2 + 1);
     V b[R2];
 #pragma unroll
     for (int t = 0; t < R2; ++t) b[t] = sm[(u * R2 + t) * W + l];

@@ -63,10 +63,10 @@ template <class P> struct Geo8 {
 // ymap.m[j]: Y of solve j as a 2-D tensor of 8-byte elements, dims
 // {M2, planes * n1}, box {16, n1}.  SHARED: every solve of the launch has the
 // same spectrum (densities of one plan); a CTA then takes one column tile for
-// all solves in turn and loads the tile's spectrum values once.
+// `run` solves in turn and loads the tile's spectrum values once.
 template <class P, int NJ, bool SHARED = false>
 __global__ void __launch_bounds__(Geo2<P>::NT, Geo2<P>::MINB_MID)
-    k8_col_mid(const Jobs jobs, int M2, int planes, const __grid_constant__ TmapSet<NJ> ymap) {
+    k8_col_mid(const Jobs jobs, int M2, int planes, int run, const __grid_constant__ TmapSet<NJ> ymap) {
   using V = float2;
   using G = Geo8<P>;
   constexpr int M = P::M, n = M / 2, W = G::W, R2 = P::R2;
@@ -87,10 +87,10 @@ __global__ void __launch_bounds__(Geo2<P>::NT, Geo2<P>::MINB_MID)
   auto job_of = [&](long long it) -> long long { return SHARED ? phys(it) % K : phys(it) / tpj; };
   auto lt_of = [&](long long it) -> long long { return SHARED ? phys(it) / K : phys(it) % tpj; };
   auto next_of = [&](long long it) -> long long {
-    if constexpr (SHARED) return it % K + 1 < K ? it + 1 : (it / K + gridDim.x) * K;
+    if constexpr (SHARED) return it % run + 1 < run ? it + 1 : (it / run + gridDim.x) * run;
     else return it + gridDim.x;
   };
-  const long long first = SHARED ? (long long)blockIdx.x * K : (long long)blockIdx.x;
+  const long long first = SHARED ? (long long)blockIdx.x * run : (long long)blockIdx.x;
   auto issue = [&](long long it) {  // thread 0
     const long long lt = lt_of(it);
     fence_proxy_async_smem();
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(Geo2<P>::NT, Geo2<P>::MINB_MID)
     // every thread has taken the tile out of the staging buffer: the next one
     if (threadIdx.x == 0 && next_of(it) < total) issue(next_of(it));
     // SHARED: the first solve of the tile this CTA takes in turn loads the spectrum
-    if (!SHARED || it % K == 0) mid_load<P>(sp, srow, u, true, n2 + 1);
+    if (!SHARED || it % run == 0) mid_load<P>(sp, srow, u, true, n2 + 1);
     V b[R2];
 #pragma unroll
     for (int t = 0; t < R2; ++t) b[t] = sm[(u * R2 + t) * W + l];
@@ -219,7 +219,7 @@ template <class P> __device__ __forceinline__ void mid8_apply(float2* b, const M
 // CTA per tile (SHARED: per tile of one solve), handed out by the queue.
 template <class P, int NJ, bool SHARED = false>
 __global__ void __launch_bounds__(Geo8W<P>::NT, Geo8W<P>::MINB)
-    k8w_col_mid(const Jobs jobs, int M2, int planes, const __grid_constant__ TmapSet<NJ> ymap) {
+    k8w_col_mid(const Jobs jobs, int M2, int planes, int, const __grid_constant__ TmapSet<NJ> ymap) {
   using V = float2;
   using G = Geo8W<P>;
   constexpr int M = P::M, n = M / 2, W = G::W, R2 = P::R2, PITCH = G::PITCH;

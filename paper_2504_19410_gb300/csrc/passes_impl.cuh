@@ -268,7 +268,7 @@ template <int M> struct Inst2 {
     const long long tiles = (long long)((M2 + W - 1) / W) * planes * jobs.count;
     constexpr int smem = G::SM_STRIDED + Stage2<P>::BYTES;
     auto f = k2p_col_mid<P>;
-    f<<<persistent_grid((const void*)f, G::NT, smem, tiles), G::NT, smem, s>>>(jobs, M2, planes);
+    f<<<persistent_grid((const void*)f, G::NT, smem, tiles), G::NT, smem, s>>>(jobs, M2, planes, 1);
     return cudaGetLastError();
   }
   static cudaError_t rowi(const Jobs& jobs, long long rows, cudaStream_t s) {
@@ -296,14 +296,16 @@ template <int M> struct Inst2 {
     const long long tiles = (long long)((M2 + W - 1) / W) * planes;
     constexpr int smem = G::SM_STRIDED + Stage2<P>::BYTES;
     auto f = k2p_col_mid<P, kMulSpectrum, true>;
-    f<<<persistent_grid((const void*)f, G::NT, smem, tiles), G::NT, smem, s>>>(jobs, M2, planes);
+    const int run = shared_run((const void*)f, G::NT, smem, tiles, jobs.count);
+    f<<<persistent_grid((const void*)f, G::NT, smem, tiles * jobs.count / run), G::NT, smem, s>>>(jobs, M2, planes,
+                                                                                                    run);
     return cudaGetLastError();
   }
   static cudaError_t colm_p_ddi(const Jobs& jobs, int M2, int planes, cudaStream_t s) {
     const long long tiles = (long long)((M2 + W - 1) / W) * planes * jobs.count;
     constexpr int smem = G::SM_STRIDED + Stage2<P>::BYTES;
     auto f = k2p_col_mid<P, kMulDdiKernel>;
-    f<<<persistent_grid((const void*)f, G::NT, smem, tiles), G::NT, smem, s>>>(jobs, M2, planes);
+    f<<<persistent_grid((const void*)f, G::NT, smem, tiles), G::NT, smem, s>>>(jobs, M2, planes, 1);
     return cudaGetLastError();
   }
   static cudaError_t c2r_epi(const Jobs& jobs, long long C, cudaStream_t s) {
@@ -426,17 +428,21 @@ static cudaError_t init_tu_twiddles() {
 #define FSA_REG_V1(ARITH, V, M) fsa::register_pass_fns(ARITH, M, fsa::fns_of<fsa::detail::Inst<V, M>>());
 #define FSA_REG_V2(M)                                                                 \
   {                                                                                   \
-    /* densities of one plan: the prefetching middle pass, whichever the     */      \
-    /* tuner picks for single solves (it overlaps loads across the densities) */     \
+    /* densities of one plan: the tensor-copy middle pass (its results equal */      \
+    /* generation 2's) or else the prefetching one, whichever the tuner picks */    \
+    /* for single solves: both overlap loads across the densities             */    \
     fsa::PassFns f2 = fsa::fns_of<fsa::detail::Inst2<M>>();                           \
-    f2.colm_shared = &fsa::detail::Inst2<M>::colm_p_shared;                           \
+    f2.colm_shared = fsa::k8_colm_shared_exact(M);                                    \
+    if (!f2.colm_shared) f2.colm_shared = &fsa::detail::Inst2<M>::colm_p_shared;      \
     fsa::register_pass_fns(fsa::kArithF32G2, M, f2);                                  \
   }                                                                                   \
   {                                                                                   \
     fsa::PassFns f3 = fsa::fns_of<fsa::detail::Inst2<M>>();                           \
     f3.colm = &fsa::detail::Inst2<M>::colm_p;                                         \
     f3.colm_ddi = &fsa::detail::Inst2<M>::colm_p_ddi;                                 \
-    f3.colm_shared = &fsa::detail::Inst2<M>::colm_p_shared;                           \
+    f3.colm_shared_p = &fsa::detail::Inst2<M>::colm_p_shared;                         \
+    f3.colm_shared = fsa::k8_colm_shared_exact(M);                                    \
+    if (!f3.colm_shared) f3.colm_shared = &fsa::detail::Inst2<M>::colm_p_shared;      \
     f3.rowf = &fsa::detail::Inst2<M>::rowf_p;                                         \
     f3.rowi = &fsa::detail::Inst2<M>::rowi_p;                                         \
     fsa::register_pass_fns(fsa::kArithF32G3, M, f3);                                  \

@@ -98,6 +98,16 @@ int persistent_grid(const void* func, int threads, int smem, long long tiles) {
   return (int)(g < 1 ? 1 : g);
 }
 
+int shared_run(const void* func, int threads, int smem, long long tiles, int count) {
+  const long long cap = persistent_grid(func, threads, smem, 1LL << 40);
+  for (int run = count; run > 1; --run) {
+    if (count % run != 0) continue;
+    const long long runs = tiles * (count / run), rounds = (runs + cap - 1) / cap;
+    if (10 * runs >= 9 * rounds * cap) return run;
+  }
+  return 1;
+}
+
 int& autotune_mode() {
   static int mode = 1;
   return mode;
