@@ -221,34 +221,6 @@ __global__ void k_t1_octant(double* __restrict__ O, int kernel, int n0, int n1, 
   }
 }
 
-// u[q] = hv U^eps(b sqrt(q)) for q < nu, w[q] = W(c sqrt(q)) for q < nw.  All
-// points of one q share its rounding error, which the DCT would then average
-// less than per-point errors; so for the 3-D Coulomb kernel the algebraic part
-// f / sqrt(q), f = hv / (4 pi b) = fh + fl, is formed to twice the working
-// precision and rounded once.
-__device__ double w_from_table(const double* __restrict__ tab, int P, double k);
-__global__ void k_radial_tables(double* __restrict__ u, long long nu, double b, double hv, double fh, double fl,
-                                double* __restrict__ w,
-                                long long nw, double c, int kernel, double eps, double lam,
-                                const double* __restrict__ wtab, int wpanels) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nu + nw;
-       i += (long long)gridDim.x * blockDim.x) {
-    if (i < nu) {
-      const double s = sqrt((double)i);
-      if (kernel == FSA_KERNEL_COULOMB3D && i > 0) {
-        const double ds = fma(-s, s, (double)i) / (2.0 * s);  // sqrt(i) = s + ds
-        const double t = fh / s;
-        u[i] = erf(b * s / eps) * (t + (fma(-t, s, fh) + (fl - t * ds)) / s);
-      } else {
-        u[i] = hv * smooth_U(kernel, b * s, eps, lam);
-      }
-    } else {
-      const double q = (double)(i - nu);
-      w[i - nu] = wtab ? w_from_table(wtab, wpanels, c * sqrt(q)) : singular_W(kernel, c * c * q, eps * eps, lam);
-    }
-  }
-}
-
 // W(k) from the quadrature table of radial_w.cpp: the panel holding k (binary
 // search over the edges), then its Chebyshev series by Clenshaw's recurrence.
 __device__ double w_from_table(const double* __restrict__ tab, int P, double k) {
@@ -269,6 +241,32 @@ __device__ double w_from_table(const double* __restrict__ tab, int P, double k) 
     b1 = b0;
   }
   return fma(t, b1, c[0] - b2);
+}
+
+// u[q] = hv U^eps(b sqrt(q)) for q < nu, w[q] = W(c sqrt(q)) for q < nw.  All
+// points of one q share its rounding error, which the DCT would then average
+// less than per-point errors; so for the 3-D Coulomb kernel the algebraic part
+// f / sqrt(q), f = hv / (4 pi b) = fh + fl, is formed to twice the working
+// precision and rounded once.
+__global__ void k_radial_tables(double* __restrict__ u, long long nu, double b, double hv, double fh, double fl,
+                                double* __restrict__ w, long long nw, double c, int kernel, double eps, double lam,
+                                const double* __restrict__ wtab, int wpanels) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nu + nw;
+       i += (long long)gridDim.x * blockDim.x) {
+    if (i < nu) {
+      const double s = sqrt((double)i);
+      if (kernel == FSA_KERNEL_COULOMB3D && i > 0) {
+        const double ds = fma(-s, s, (double)i) / (2.0 * s);  // sqrt(i) = s + ds
+        const double t = fh / s;
+        u[i] = erf(b * s / eps) * (t + (fma(-t, s, fh) + (fl - t * ds)) / s);
+      } else {
+        u[i] = hv * smooth_U(kernel, b * s, eps, lam);
+      }
+    } else {
+      const double q = (double)(i - nu);
+      w[i - nu] = wtab ? w_from_table(wtab, wpanels, c * sqrt(q)) : singular_W(kernel, c * c * q, eps * eps, lam);
+    }
+  }
 }
 
 template <typename R>
