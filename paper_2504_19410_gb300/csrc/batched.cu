@@ -34,6 +34,7 @@ struct GroupKey {
   }
 };
 
+constexpr size_t kSigHead = 2;  // entries of a signature before its plans
 struct Sig {
   std::vector<const void*> v;
   bool operator<(const Sig& o) const { return v < o.v; }
@@ -299,11 +300,12 @@ void batched_forget_plan(const fsa_plan* p) {
     DeviceCtx& c = dc.second;
     for (auto it = c.lru.begin(); it != c.lru.end();) {
       bool uses = false;
-      for (size_t i = 1; i < it->v.size(); i += 3) uses |= (it->v[i] == p);  // v = mode, then (plan, rho, phi)...
+      // v = mode, selection generation, then (plan, rho, phi)...
+      for (size_t i = kSigHead; i < it->v.size(); i += 3) uses |= (it->v[i] == p);
       if (uses) {
         cudaGraphExecDestroy(c.graphs[*it]);
         std::vector<const void*> pkey;
-        for (size_t i = 1; i < it->v.size(); i += 3) pkey.push_back(it->v[i]);
+        for (size_t i = kSigHead; i < it->v.size(); i += 3) pkey.push_back(it->v[i]);
         g_choice.erase(pkey);
         c.graphs.erase(*it);
         it = c.lru.erase(it);
