@@ -72,8 +72,8 @@ __device__ __forceinline__ void dct_stages(int t, double2* sm, const Ld& ld, con
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const int p = b + r * NS, q = b % R0;
-          if (p <= P::M / 2) st(p, v[k][r]);
-          else if (P::NST > 1 && q != 0 && q != R0 / 2) st(P::M - p, v[k][r]);
+          const bool lo = p <= P::M / 2;
+          if (lo || (P::NST > 1 && q != 0 && q != R0 / 2)) st(lo ? p : P::M - p, v[k][r]);
         }
       } else if constexpr (S == 0) {
 #pragma unroll

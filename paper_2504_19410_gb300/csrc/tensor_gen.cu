@@ -309,7 +309,9 @@ namespace {
 // One DCT pass: the octant in place, from the U table, or to the spectrum.
 template <int M> struct DctInst {
   using P = typename PlanFor<M>::type;
-  static constexpr int W = 8;
+  // line pairs per CTA; lengths 48 and 64 in CTAs of about one warp: a 32^3
+  // octant's 545 pairs then spread over 137 SMs' FP64 pipes, not 69
+  static constexpr int W = M == 48 || M == 64 ? 4 : 8;
   static constexpr int T = threads_per_line<P, W>();
   static constexpr int SM = smem_strided<P, double2, W>();
   template <class Src, class Dst> static cudaError_t set() {
