@@ -134,14 +134,15 @@ struct DctRadial {
     return __ldg(tab + ra * a * a + rb * b * b + re * m * m);
   }
 };
-// The stored spectrum: (X + W) norm, W from its table.
+// The stored spectrum: (X + W) norm, W from its table (the sum rounded by
+// itself, as where X is read back: the two forms agree bit for bit).
 template <typename R> struct DctSpectrum {
   R* S;
   DctArray idx;
   DctRadial w;
   double norm;
   __device__ __forceinline__ void operator()(int a, int b, int p, double v) const {
-    S[idx.at(a, b, p)] = (R)((v + w(a, b, p)) * norm);
+    S[idx.at(a, b, p)] = (R)(__dadd_rn(v, w(a, b, p)) * norm);
   }
 };
 

@@ -227,7 +227,8 @@ cudaError_t noalloc_resolve(int dev);
 cudaError_t tensorgen_init_twiddles();
 // param: the kernel's parameter (the Yukawa lam), ignored by the others.
 // utab_mem, wtab_mem: room for a quarter of the octant's points in doubles
-// each (tables of U^eps and W, used until the call's work ends), or null.
+// each (tables of U^eps and W, used until the call's work ends), or null (the
+// same values, evaluated per point).
 cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], double eps, double param,
                           double* oct64, void* out, fsa_dtype dtype, cudaStream_t s,
                           const double* wtab = nullptr, int wtab_panels = 0, double* utab_mem = nullptr,

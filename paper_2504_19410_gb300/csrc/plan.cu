@@ -1240,7 +1240,7 @@ fsa_status attach_w_table(fsa_plan* p) {
 // otherwise: FP64 plans the double-word copy's, before it is made; FP32 plans
 // the spectrum's for U^eps (written only by the last pass) and, for W, what the
 // scratch holds beyond the octant (a plan's workspace does; a serving plan's
-// scratch does not, and evaluates W per point).
+// scratch does not, and evaluates the same W per point).
 cudaError_t plan_generate_into(fsa_plan* p, void* scratch, size_t scratch_bytes, cudaStream_t s) {
   double* oct = p->dtype == FSA_F64 ? (double*)p->spectrum : (double*)scratch;
   const size_t total = octant_count(p->n, p->d), quarter = align256(total / 4 * 8);

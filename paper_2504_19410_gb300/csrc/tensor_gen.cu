@@ -48,8 +48,10 @@
 // the octant.  Measured (GB300, FP64 plan of 256^3): octant
 // 2.60 and spectrum 0.89 ms before, 0.11 ms for the tables now; with the
 // pruned DCT passes the whole generation 6.65 -> 2.00 ms.
-// Other grids (no common integer ratio, or a table above a quarter of the
-// octant: planes, very flat boxes) evaluate per point.
+// Where there is no memory for a table (a serving plan's W) the same function
+// of q is evaluated per point, with the same bits.  Other grids (no common
+// integer ratio, or a table above a quarter of the octant: planes, very flat
+// boxes) evaluate per point, from the sum of squares.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -205,8 +207,49 @@ __device__ __forceinline__ double smooth_U(int kernel, double r, double eps, dou
   }
 }
 
+// A radial function's integer argument: q = ra a^2 + rb b^2 + rc c^2.
+struct RadialArg {
+  int ra, rb, rc;
+  __device__ __forceinline__ double operator()(int a, int b, int c) const {
+    return (double)(ra * a * a + rb * b * b + rc * c * c);
+  }
+};
+// hv U^eps(b sqrt(q)).  All points of one q share its rounding error, which the
+// DCT would then average less than per-point errors; so for the 3-D Coulomb
+// kernel the algebraic part f / sqrt(q), f = hv / (4 pi b) = fh + fl, is formed
+// to twice the working precision and rounded once.
+struct RadialU {
+  double b, hv, fh, fl, eps, lam;
+  int kernel;
+};
+// W(c sqrt(q))
+struct RadialW {
+  double c, eps, lam;
+  const double* tab;
+  int panels, kernel;
+};
+__device__ double w_from_table(const double* __restrict__ tab, int P, double k);
+// Not inlined: the tables and the per-point kernels then run the same
+// instructions (inlined, the compiler fuses products into whatever sum follows
+// them), so a plan's spectrum does not depend on which of the two its memory
+// allowed.
+__device__ __noinline__ double radial_U(const RadialU& u, double q) {
+  const double s = sqrt(q);
+  if (u.kernel == FSA_KERNEL_COULOMB3D && q > 0.0) {
+    const double ds = fma(-s, s, q) / (2.0 * s);  // sqrt(q) = s + ds
+    const double t = u.fh / s;
+    return erf(u.b * s / u.eps) * (t + (fma(-t, s, u.fh) + (u.fl - t * ds)) / s);
+  }
+  return u.hv * smooth_U(u.kernel, u.b * s, u.eps, u.lam);
+}
+__device__ __noinline__ double radial_W(const RadialW& w, double q) {
+  return w.tab ? w_from_table(w.tab, w.panels, w.c * sqrt(q)) : singular_W(w.kernel, w.c * w.c * q, w.eps * w.eps, w.lam);
+}
+
+// RADIAL: through the integer argument, as the table would hold it.
+template <bool RADIAL>
 __global__ void k_t1_octant(double* __restrict__ O, int kernel, int n0, int n1, int n2, double h0, double h1,
-                            double h2, double eps, double lam) {
+                            double h2, double eps, double lam, RadialArg arg, const __grid_constant__ RadialU u) {
   const long long total = (long long)(n0 + 1) * (n1 + 1) * (n2 + 1);
   const double hv = h0 * h1 * h2;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -215,6 +258,10 @@ __global__ void k_t1_octant(double* __restrict__ O, int kernel, int n0, int n1, 
     const long long r01 = i / (n2 + 1);
     const int p1 = (int)(r01 % (n1 + 1));
     const int p0 = (int)(r01 / (n1 + 1));
+    if constexpr (RADIAL) {
+      O[i] = radial_U(u, arg(p0, p1, p2));
+      continue;
+    }
     const double x = p0 * h0, y = p1 * h1, z = p2 * h2;
     const double r = sqrt(x * x + y * y + z * z);
     O[i] = hv * smooth_U(kernel, r, eps, lam);
@@ -243,37 +290,22 @@ __device__ double w_from_table(const double* __restrict__ tab, int P, double k) 
   return fma(t, b1, c[0] - b2);
 }
 
-// u[q] = hv U^eps(b sqrt(q)) for q < nu, w[q] = W(c sqrt(q)) for q < nw.  All
-// points of one q share its rounding error, which the DCT would then average
-// less than per-point errors; so for the 3-D Coulomb kernel the algebraic part
-// f / sqrt(q), f = hv / (4 pi b) = fh + fl, is formed to twice the working
-// precision and rounded once.
-__global__ void k_radial_tables(double* __restrict__ u, long long nu, double b, double hv, double fh, double fl,
-                                double* __restrict__ w, long long nw, double c, int kernel, double eps, double lam,
-                                const double* __restrict__ wtab, int wpanels) {
+// tu[q] = hv U^eps(b sqrt(q)) for q < nu, tw[q] = W(c sqrt(q)) for q < nw.
+__global__ void k_radial_tables(double* __restrict__ tu, long long nu, double* __restrict__ tw, long long nw,
+                                const __grid_constant__ RadialU u, const __grid_constant__ RadialW w) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nu + nw;
        i += (long long)gridDim.x * blockDim.x) {
-    if (i < nu) {
-      const double s = sqrt((double)i);
-      if (kernel == FSA_KERNEL_COULOMB3D && i > 0) {
-        const double ds = fma(-s, s, (double)i) / (2.0 * s);  // sqrt(i) = s + ds
-        const double t = fh / s;
-        u[i] = erf(b * s / eps) * (t + (fma(-t, s, fh) + (fl - t * ds)) / s);
-      } else {
-        u[i] = hv * smooth_U(kernel, b * s, eps, lam);
-      }
-    } else {
-      const double q = (double)(i - nu);
-      w[i - nu] = wtab ? w_from_table(wtab, wpanels, c * sqrt(q)) : singular_W(kernel, c * c * q, eps * eps, lam);
-    }
+    if (i < nu) tu[i] = radial_U(u, (double)i);
+    else tw[i - nu] = radial_W(w, (double)(i - nu));
   }
 }
 
-template <typename R>
+template <typename R, bool RADIAL>
 __global__ void k_spectrum_finalize(const double* S1, R* S,  // may alias (FP64 plans)
                                     int kernel, int n0, int n1, int n2,
                                     double c0, double c1, double c2, double eps, double lam, double inv_norm,
-                                    const double* __restrict__ wtab, int wpanels) {
+                                    const double* __restrict__ wtab, int wpanels, RadialArg arg,
+                                    const __grid_constant__ RadialW rw) {
   const long long total = (long long)(n0 + 1) * (n1 + 1) * (n2 + 1);
   const double e2 = eps * eps;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -282,6 +314,10 @@ __global__ void k_spectrum_finalize(const double* S1, R* S,  // may alias (FP64 
     const long long r01 = i / (n2 + 1);
     const int p1 = (int)(r01 % (n1 + 1));
     const int p0 = (int)(r01 / (n1 + 1));
+    if constexpr (RADIAL) {
+      S[i] = (R)((S1[i] + radial_W(rw, arg(p0, p1, p2))) * inv_norm);
+      continue;
+    }
     const double m0 = c0 * p0, m1 = c1 * p1, m2 = c2 * p2;  // mu_j = pi p_j / (2 L_j)
     const double k2 = m0 * m0 + m1 * m1 + m2 * m2;
     const double w = wtab ? w_from_table(wtab, wpanels, sqrt(k2)) : singular_W(kernel, k2, e2, lam);
@@ -436,20 +472,25 @@ cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], 
   const double inv_norm = plane ? 1.0 / (4.0 * (double)n0 * n1) : 1.0 / (8.0 * (double)n0 * n1 * n2);
   const double c2 = plane ? 0.0 : pi / (2 * L[2]);
   const double hs[3] = {h0, h1, h2}, cs[3] = {pi / (2 * L[0]), pi / (2 * L[1]), c2};
+  // Whether the functions are radial in this sense is the grid's property alone;
+  // the tables take the memory there is, and without it the same values are
+  // evaluated per point.
   Radial ru{}, rw{};
-  const bool tu = !plane && utab_mem && radial_of(hs, n, total, &ru);
-  const bool tw = !plane && wtab_mem && radial_of(cs, n, total, &rw);
+  const bool hu = !plane && radial_of(hs, n, total, &ru), hw = !plane && radial_of(cs, n, total, &rw);
+  const bool tu = hu && utab_mem, tw = hw && wtab_mem;
+  const long double f = hu ? (long double)h0 * h1 * h2 / (4.0L * 3.141592653589793238462643383279502884L * ru.base) : 0.0L;
+  const RadialU fu{ru.base, h0 * h1 * h2, (double)f, (double)(f - (long double)(double)f), eps, lam, (int)kernel};
+  const RadialW fw{rw.base, eps, lam, wtab, wtab_panels, (int)kernel};
+  const RadialArg au{ru.r[0], ru.r[1], ru.r[2]}, aw{rw.r[0], rw.r[1], rw.r[2]};
   cudaError_t e = cudaSuccess;
   if (tu || tw) {
     const long long nu = tu ? ru.size : 0, nw = tw ? rw.size : 0;
-    const long double f = (long double)h0 * h1 * h2 / (4.0L * 3.141592653589793238462643383279502884L * ru.base);
-    const double fh = tu ? (double)f : 0.0, fl = tu ? (double)(f - (long double)fh) : 0.0;
-    k_radial_tables<<<blocks_for(nu + nw), threads, 0, s>>>(utab_mem, nu, ru.base, h0 * h1 * h2, fh, fl, wtab_mem, nw,
-                                                            rw.base, (int)kernel, eps, lam, wtab, wtab_panels);
+    k_radial_tables<<<blocks_for(nu + nw), threads, 0, s>>>(utab_mem, nu, wtab_mem, nw, fu, fw);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && !tu) {
-    k_t1_octant<<<blocks_for(total), threads, 0, s>>>(O, (int)kernel, n0, n1, n2, h0, h1, h2, eps, lam);
+    (hu ? k_t1_octant<true> : k_t1_octant<false>)<<<blocks_for(total), threads, 0, s>>>(
+        O, (int)kernel, n0, n1, n2, h0, h1, h2, eps, lam, au, fu);
     e = cudaGetLastError();
   }
   // axis 2: lines (p0, p1), element stride 1
@@ -468,12 +509,12 @@ cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], 
         : dtype == FSA_F64 ? dct_run(2 * n0, x0, DctSpectrum<double>{(double*)out, x0, w0, inv_norm}, e1 * e2, e2, s)
                            : dct_run(2 * n0, x0, DctSpectrum<float>{(float*)out, x0, w0, inv_norm}, e1 * e2, e2, s);
   if (e != cudaSuccess || tw) return e;
-  if (dtype == FSA_F64)
-    k_spectrum_finalize<double><<<blocks_for(total), threads, 0, s>>>(O, (double*)out, (int)kernel, n0, n1, n2, cs[0],
-                                                                      cs[1], c2, eps, lam, inv_norm, wtab, wtab_panels);
-  else
-    k_spectrum_finalize<float><<<blocks_for(total), threads, 0, s>>>(O, (float*)out, (int)kernel, n0, n1, n2, cs[0],
-                                                                     cs[1], c2, eps, lam, inv_norm, wtab, wtab_panels);
+  auto finalize = [&](auto kern, auto* S) {
+    kern<<<blocks_for(total), threads, 0, s>>>(O, S, (int)kernel, n0, n1, n2, cs[0], cs[1], c2, eps, lam, inv_norm, wtab,
+                                               wtab_panels, aw, fw);
+  };
+  if (dtype == FSA_F64) finalize(hw ? k_spectrum_finalize<double, true> : k_spectrum_finalize<double, false>, (double*)out);
+  else finalize(hw ? k_spectrum_finalize<float, true> : k_spectrum_finalize<float, false>, (float*)out);
   return cudaGetLastError();
 }
 
