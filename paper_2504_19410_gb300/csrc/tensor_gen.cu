@@ -59,6 +59,7 @@
 #include "dct.cuh"
 #include "fsa_internal.h"
 #include "quad.h"
+#include "radial.h"
 
 namespace fsa {
 
@@ -402,37 +403,6 @@ cudaError_t dct_run(int M, const Src& src, const Dst& dst, long long nlines, lon
 
 #undef FSA_DCT_DISPATCH
 
-// The integers r_j with s_j^2 = base^2 r_j (to round-off) and the table length
-// sum_j r_j n_j^2 + 1; false where no base s_min / m, m <= 3, gives integers or
-// the table would hold more than a quarter of the octant's points (more
-// evaluations saved than made, and room for two tables in the octant).
-struct Radial {
-  double base;
-  int r[3];
-  long long size;
-};
-bool radial_of(const double* sj, const int* n, long long total, Radial* out) {
-  const double lo = std::min(sj[0], std::min(sj[1], sj[2]));
-  for (int m = 1; m <= 3; ++m) {
-    out->base = lo / m;
-    long long size = 1;
-    bool ok = true;
-    for (int j = 0; j < 3 && ok; ++j) {
-      const double x = sj[j] / lo, v = x * x * (m * m), rv = std::nearbyint(v);
-      ok = std::fabs(v - rv) <= 4e-15 * rv && rv * n[j] * n[j] < 1e9;
-      if (ok) {
-        out->r[j] = (int)rv;
-        size += (long long)rv * n[j] * n[j];
-      }
-    }
-    if (ok && size <= total / 4) {
-      out->size = size;
-      return true;
-    }
-  }
-  return false;
-}
-
 }  // namespace
 
 cudaError_t tensorgen_prepare(int M) { return dct_prepare(M); }
@@ -472,11 +442,13 @@ cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], 
   const double inv_norm = plane ? 1.0 / (4.0 * (double)n0 * n1) : 1.0 / (8.0 * (double)n0 * n1 * n2);
   const double c2 = plane ? 0.0 : pi / (2 * L[2]);
   const double hs[3] = {h0, h1, h2}, cs[3] = {pi / (2 * L[0]), pi / (2 * L[1]), c2};
+  const long double hx[3] = {(long double)L[0] / n0, (long double)L[1] / n1, plane ? 1.0L : (long double)L[2] / n2};
+  const long double cx[3] = {1.0L / L[0], 1.0L / L[1], plane ? 1.0L : 1.0L / L[2]};
   // Whether the functions are radial in this sense is the grid's property alone;
   // the tables take the memory there is, and without it the same values are
   // evaluated per point.
   Radial ru{}, rw{};
-  const bool hu = !plane && radial_of(hs, n, total, &ru), hw = !plane && radial_of(cs, n, total, &rw);
+  const bool hu = !plane && radial_of(hs, hx, n, total, &ru), hw = !plane && radial_of(cs, cx, n, total, &rw);
   const bool tu = hu && utab_mem, tw = hw && wtab_mem;
   const long double f = hu ? (long double)h0 * h1 * h2 / (4.0L * 3.141592653589793238462643383279502884L * ru.base) : 0.0L;
   const RadialU fu{ru.base, h0 * h1 * h2, (double)f, (double)(f - (long double)(double)f), eps, lam, (int)kernel};
