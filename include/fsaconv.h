@@ -198,7 +198,12 @@ fsa_status fsa_plan_create_ddi3d(fsa_plan** out, const double* L, const int* n, 
  * S[p] = (DFT_{2n}(T^(1))[p] + W(|mu_p|)) / (8 n0 n1 n2) for p_j in [0, n_j];
  * T is real and even per axis (Sec. 2.3), so this octant is the whole
  * spectrum.  The DFT of the even tensor is a separable DCT-I, computed with
- * the library's FFT kernels.  Asynchronous on stream; idempotent. */
+ * the library's FFT kernels.  Asynchronous on stream; idempotent: generating
+ * a plan again stores the same values.  FP32 plans use their workspace as the
+ * FP64 scratch and native-FP64 plans (fsa_plan_info.arithmetic 1) build the
+ * spectrum where it is stored, so order a plan's solves after it; a solve that
+ * uses neither (fsa_apply_noalloc of an FP32 plan, solves of a double-word
+ * plan) reads the same values while the plan is generated again. */
 fsa_status fsa_tensor_generate(fsa_plan* plan, fsa_stream_t stream);
 
 /* Phi = T * rho (Eq. DiscConv) by zero-padding to 2n per axis, FFT, multiply

@@ -226,13 +226,15 @@ cudaError_t tensorgen_prepare(int M);
 cudaError_t noalloc_resolve(int dev);
 cudaError_t tensorgen_init_twiddles();
 // param: the kernel's parameter (the Yukawa lam), ignored by the others.
-// utab_mem, wtab_mem: room for a quarter of the octant's points in doubles
-// each (tables of U^eps and W, used until the call's work ends), or null (the
-// same values, evaluated per point).
+// utab_mem, wtab_mem: room for the radial tables of U^eps and W
+// (tensorgen_tables; at most a quarter of the octant's points each), used until
+// the call's work ends, or null (the same values, evaluated per point).
 cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], double eps, double param,
                           double* oct64, void* out, fsa_dtype dtype, cudaStream_t s,
                           const double* wtab = nullptr, int wtab_panels = 0, double* utab_mem = nullptr,
                           double* wtab_mem = nullptr);
+// Entries of those tables for a grid of d = 3 (0: the function has none there).
+void tensorgen_tables(const int n[3], const double L[3], long long* u, long long* w);
 
 // Twiddle table exp(-2 pi i k / 3072), k < 3072, computed on the host.
 void host_twiddles(double* re, double* im);
@@ -259,6 +261,11 @@ struct fsa_plan {
   void* spectrum;
   size_t spectrum_bytes;
   void* spectrum_dw;  // FP64 plans: the spectrum as double-word pairs
+  // FP64 plans with a workspace: room for generation's radial tables (behind
+  // spectrum_dw, in its allocation; null where there was none), U^eps's taking
+  // gen_tab_u bytes
+  double* gen_tab;
+  size_t gen_tab_u;
   int f64_dw;         // FP64 plans: 1 = double-word arithmetic, 0 = native FP64
   long long chunk_bytes;  // pass split: target bytes of one slab's X + Y (<= 0: no split)
   void* ws;  // X then Y (then, for DDI plans, the host path's staging of rho)

@@ -930,7 +930,22 @@ fsa_status plan_create_core(fsa_plan** out, fsa_kernel kernel, const double* L, 
   p->ws_bytes = with_workspace ? plan_workspace_bytes(n, dtype) + extra_ws : 0;
   // The workspace always holds the FP64 generation scratch of an FP32 plan.
   e = cudaMalloc(&p->spectrum, p->spectrum_bytes);
-  if (e == cudaSuccess && dtype == FSA_F64) e = cudaMalloc(&p->spectrum_dw, p->spectrum_bytes);
+  if (e == cudaSuccess && dtype == FSA_F64) {
+    // generation's tables behind it, where memory allows (at most half the
+    // octant's points; a cube's take 2 % at 256^3).  A serving plan is
+    // generated once, before anything reads it: its tables lie in spectrum_dw.
+    long long nu = 0, nw = 0;
+    if (with_workspace && d == 3) tensorgen_tables(n, L, &nu, &nw);
+    const size_t off = align256(p->spectrum_bytes), ub = align256((size_t)nu * 8), wb = align256((size_t)nw * 8);
+    if (ub + wb > 0 && cudaMalloc(&p->spectrum_dw, off + ub + wb) == cudaSuccess) {
+      p->gen_tab = (double*)((char*)p->spectrum_dw + off);
+      p->gen_tab_u = ub;
+    } else {
+      cudaGetLastError();
+      p->spectrum_dw = nullptr;
+      e = cudaMalloc(&p->spectrum_dw, p->spectrum_bytes);
+    }
+  }
   if (e == cudaSuccess && with_workspace) e = cudaMalloc(&p->ws, p->ws_bytes);
   if (e != cudaSuccess) {
     if (p->spectrum) cudaFree(p->spectrum);
@@ -1236,22 +1251,33 @@ fsa_status attach_w_table(fsa_plan* p) {
 }
 
 // scratch, scratch_bytes: FP32 plans: at least plan_gen_scratch_bytes.  The
-// radial tables (tensor_gen.cu) take memory the generation does not use
-// otherwise: FP64 plans the double-word copy's, before it is made; FP32 plans
-// the spectrum's for U^eps (written only by the last pass) and, for W, what the
-// scratch holds beyond the octant (a plan's workspace does; a serving plan's
-// scratch does not, and evaluates the same W per point).
+// radial tables (tensor_gen.cu) lie where no solve reads: in memory of their own
+// (FP64), behind the octant in the workspace (FP32).  So generating a plan again
+// leaves its stored spectrum as it was until the same values are written over
+// it.  A plan without such memory that is generated for the first time has them
+// where the spectrum will be: FP64 plans in the double-word copy's memory, FP32
+// plans (serving plans: their scratch holds just the octant) U^eps in the
+// spectrum's, with W evaluated per point.
 cudaError_t plan_generate_into(fsa_plan* p, void* scratch, size_t scratch_bytes, cudaStream_t s) {
   double* oct = p->dtype == FSA_F64 ? (double*)p->spectrum : (double*)scratch;
   const size_t total = octant_count(p->n, p->d), quarter = align256(total / 4 * 8);
   double *ut = nullptr, *wt = nullptr;
-  if (p->dtype == FSA_F64 && p->spectrum_dw) {
-    ut = (double*)p->spectrum_dw;
-    if (2 * quarter <= total * 8) wt = (double*)((char*)p->spectrum_dw + quarter);
-  } else if (p->dtype == FSA_F32) {
-    ut = (double*)p->spectrum;
+  if (p->dtype == FSA_F64) {
+    if (p->gen_tab) {
+      ut = p->gen_tab;
+      wt = (double*)((char*)p->gen_tab + p->gen_tab_u);
+    } else if (p->spectrum_dw && !p->generated) {
+      ut = (double*)p->spectrum_dw;
+      if (2 * quarter <= total * 8) wt = (double*)((char*)p->spectrum_dw + quarter);
+    }
+  } else {
     const size_t off = align256(total * 8);
-    if (scratch_bytes >= off + quarter) wt = (double*)((char*)scratch + off);
+    if (scratch_bytes >= off + 2 * quarter) {
+      ut = (double*)((char*)scratch + off);
+      wt = (double*)((char*)scratch + off + quarter);
+    } else if (!p->generated) {
+      ut = (double*)p->spectrum;
+    }
   }
   // a DDI plan's tensor is the Coulomb kernel's (Sec. 5, Example 4)
   const fsa_kernel k = p->kernel == FSA_KERNEL_DDI3D ? FSA_KERNEL_COULOMB3D : p->kernel;

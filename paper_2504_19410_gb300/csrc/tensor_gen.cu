@@ -425,6 +425,32 @@ cudaError_t tensorgen_init_twiddles() {
   return e;
 }
 
+namespace {
+// The integer arguments of U^eps (mesh steps) and W (steps of mu) on a grid of
+// d = 3; size 0 where there is none.
+void radial_args(const int n[3], const double L[3], Radial* u, Radial* w) {
+  const double pi = 3.14159265358979323846;
+  const long long total = (long long)(n[0] + 1) * (n[1] + 1) * (n[2] + 1);
+  double hs[3], cs[3];
+  long double hx[3], cx[3];
+  for (int j = 0; j < 3; ++j) {
+    hs[j] = 2.0 * L[j] / n[j];
+    cs[j] = pi / (2 * L[j]);
+    hx[j] = (long double)L[j] / n[j];
+    cx[j] = 1.0L / L[j];
+  }
+  if (!radial_of(hs, hx, n, total, u)) *u = Radial{};
+  if (!radial_of(cs, cx, n, total, w)) *w = Radial{};
+}
+}  // namespace
+
+void tensorgen_tables(const int n[3], const double L[3], long long* u, long long* w) {
+  Radial ru, rw;
+  radial_args(n, L, &ru, &rw);
+  *u = ru.size;
+  *w = rw.size;
+}
+
 cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], double eps, double lam, double* O,
                           void* out, fsa_dtype dtype, cudaStream_t s, const double* wtab, int wtab_panels,
                           double* utab_mem, double* wtab_mem) {
@@ -441,14 +467,12 @@ cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], 
   const double pi = 3.14159265358979323846;
   const double inv_norm = plane ? 1.0 / (4.0 * (double)n0 * n1) : 1.0 / (8.0 * (double)n0 * n1 * n2);
   const double c2 = plane ? 0.0 : pi / (2 * L[2]);
-  const double hs[3] = {h0, h1, h2}, cs[3] = {pi / (2 * L[0]), pi / (2 * L[1]), c2};
-  const long double hx[3] = {(long double)L[0] / n0, (long double)L[1] / n1, plane ? 1.0L : (long double)L[2] / n2};
-  const long double cx[3] = {1.0L / L[0], 1.0L / L[1], plane ? 1.0L : 1.0L / L[2]};
   // Whether the functions are radial in this sense is the grid's property alone;
   // the tables take the memory there is, and without it the same values are
   // evaluated per point.
   Radial ru{}, rw{};
-  const bool hu = !plane && radial_of(hs, hx, n, total, &ru), hw = !plane && radial_of(cs, cx, n, total, &rw);
+  if (!plane) radial_args(n, L, &ru, &rw);
+  const bool hu = ru.size > 0, hw = rw.size > 0;
   const bool tu = hu && utab_mem, tw = hw && wtab_mem;
   const long double f = hu ? (long double)h0 * h1 * h2 / (4.0L * 3.141592653589793238462643383279502884L * ru.base) : 0.0L;
   const RadialU fu{ru.base, h0 * h1 * h2, (double)f, (double)(f - (long double)(double)f), eps, lam, (int)kernel};
@@ -482,7 +506,7 @@ cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], 
                            : dct_run(2 * n0, x0, DctSpectrum<float>{(float*)out, x0, w0, inv_norm}, e1 * e2, e2, s);
   if (e != cudaSuccess || tw) return e;
   auto finalize = [&](auto kern, auto* S) {
-    kern<<<blocks_for(total), threads, 0, s>>>(O, S, (int)kernel, n0, n1, n2, cs[0], cs[1], c2, eps, lam, inv_norm, wtab,
+    kern<<<blocks_for(total), threads, 0, s>>>(O, S, (int)kernel, n0, n1, n2, pi / (2 * L[0]), pi / (2 * L[1]), c2, eps, lam, inv_norm, wtab,
                                                wtab_panels, aw, fw);
   };
   if (dtype == FSA_F64) finalize(hw ? k_spectrum_finalize<double, true> : k_spectrum_finalize<double, false>, (double*)out);
