@@ -88,26 +88,38 @@ __device__ __forceinline__ void tile_queue_init(TileQueue* q) {
   q->next = -1;
   tile_request(q);
 }
-// thread 0: wait (bounded) for the answer to the request in flight and
-// publish it (read `next` after a barrier).  A wait that gives up ends this
-// CTA's tiles and is recorded in the fault word.
-__device__ __forceinline__ void tile_answer(TileQueue* q, unsigned parity, unsigned int* fault) {
-  int next = -1;
-  if (mbar_wait(&q->bar, parity)) {
-    unsigned ok, x;
-    asm volatile(
-        "{\n .reg .b128 r;\n .reg .pred p;\n ld.shared.b128 r, [%2];\n"
-        " clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n selp.u32 %0, 1, 0, p;\n mov.u32 %1, 0;\n"
-        " @p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n}\n"
-        : "=r"(ok), "=r"(x)
-        : "r"(smem_u32(&q->resp))
-        : "memory");
-    if (ok) next = (int)x;
-  } else {
-    if (fault) atomicOr(fault, kWaitTimeout);
-    mbar_wait(&q->bar, parity);  // the answer still in flight
+// The next tile of a CTA, -1 for none: wait() waits (bounded) for the answer
+// and tells whether it came, read() decodes it, late() records a wait that gave
+// up.  A tile that was granted is this CTA's alone, so the answer is taken
+// however late it comes; only when a second wait gives up too are there no
+// more tiles.
+template <class Wait, class Read, class Late>
+__host__ __device__ __forceinline__ int granted_tile(const Wait& wait, const Read& read, const Late& late) {
+  if (!wait()) {
+    late();
+    if (!wait()) return -1;
   }
-  q->next = next;
+  return read();
+}
+// thread 0: the answer to the request in flight, published in `next` (read it
+// after a barrier).  A wait that gives up is recorded in the fault word.
+__device__ __forceinline__ void tile_answer(TileQueue* q, unsigned parity, unsigned int* fault) {
+  q->next = granted_tile(
+      [&] { return mbar_wait(&q->bar, parity); },
+      [&]() -> int {
+        unsigned ok, x;
+        asm volatile(
+            "{\n .reg .b128 r;\n .reg .pred p;\n ld.shared.b128 r, [%2];\n"
+            " clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n selp.u32 %0, 1, 0, p;\n mov.u32 %1, 0;\n"
+            " @p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n}\n"
+            : "=r"(ok), "=r"(x)
+            : "r"(smem_u32(&q->resp))
+            : "memory");
+        return ok ? (int)x : -1;
+      },
+      [&] {
+        if (fault) atomicOr(fault, kWaitTimeout);
+      });
 }
 
 }  // namespace fsa

@@ -277,7 +277,9 @@ __global__ void __launch_bounds__(Geo8W<P>::NT, Geo8W<P>::MINB)
     if (__syncthreads_or(late)) {
       if (threadIdx.x == 0) {
         if (jobs.fault) atomicOr(jobs.fault, kWaitTimeout);
-        mbar_wait(bar, par);  // the copy and the answer still in flight
+        // the copy and the answer still in flight; a CTA that gives up leaves
+        // its tile and one it was granted undone, which the fault word says
+        mbar_wait(bar, par);
         mbar_wait(&tq->bar, qpar);
       }
       __syncthreads();
