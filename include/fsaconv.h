@@ -310,8 +310,8 @@ fsa_status fsa_apply_batched_launches(const fsa_plan* const* plans, int count, i
  * phi[k] = T * rho[k] (the plan's kernel, DDI plans included) for k < count in
  * one launch sequence: every pass is one persistent launch over the tiles of
  * all densities, and the middle pass takes a column tile for every density in
- * turn, reading the tile's spectrum values once (FP32, generations 3 and 4).
- * Results equal fsa_apply's bit for bit.  rho[k], phi[k]: device arrays as for
+ * turn, reading the tile's spectrum values once per run of densities (FP32,
+ * every generation but the first).  Results equal fsa_apply's bit for bit.  rho[k], phi[k]: device arrays as for
  * fsa_apply, 16-byte aligned; phi[k] == rho[k] is allowed, other overlaps are
  * not.  Asynchronous on stream; calls on one plan must not overlap on the GPU.
  * Errors: FSA_ERR_INVALID_ARG (count < 1 or above the capacity, NULL or

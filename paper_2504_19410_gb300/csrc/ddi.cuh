@@ -62,18 +62,12 @@ template <typename T> __device__ __forceinline__ T ddi_beta(const DdiPar* __rest
 
 // phi[0..1] = v + beta * rho[0..1] (the grid reading's -(m.n) rho term),
 // added in the precision of the output array.
-// The pair of rho values the epilogue adds, as loaded (FP64 arrays for both
-// FP64 arithmetics).
-template <typename V> struct PairOf { using T = V; };
-
-template <typename V>
-__device__ __forceinline__ typename PairOf<V>::T load_rho_pair(const typename Io<V>::T* r) {
-  return *reinterpret_cast<const typename PairOf<V>::T*>(r);
+template <typename V> __device__ __forceinline__ V load_rho_pair(const typename Io<V>::T* r) {
+  return *reinterpret_cast<const V*>(r);
 }
 
 template <typename V>
-__device__ __forceinline__ void store_pair_axpy(typename Io<V>::T* p, V v, typename Io<V>::T beta,
-                                                typename PairOf<V>::T a) {
+__device__ __forceinline__ void store_pair_axpy(typename Io<V>::T* p, V v, typename Io<V>::T beta, V a) {
   *reinterpret_cast<V*>(p) = mk(v.x + beta * a.x, v.y + beta * a.y);
 }
 

@@ -38,11 +38,6 @@ __device__ __forceinline__ dw dw_two_sum(float a, float b) {
   return dw(s, e);
 }
 
-__device__ __forceinline__ dw dw_fast_two_sum(float a, float b) {  // |a| >= |b| or a == 0
-  const float s = __fadd_rn(a, b);
-  return dw(s, __fsub_rn(b, __fsub_rn(s, a)));
-}
-
 __device__ __forceinline__ dw operator+(dw x, dw y) {
   const dw s = dw_two_sum(x.hi, y.hi);
   return dw(s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo)));

@@ -180,6 +180,13 @@ int shared_run(const void* func, int threads, int smem, long long tiles, int cou
 // (resident CTAs x SMs, the default), 1 = one CTA per tile, so that the
 // blocks of a long solve retire one tile at a time and kernels of
 // higher-priority streams get SMs between them (the serving loop's bulk lane).
+// The kernels with a tile queue (mbar.cuh: the double-word passes, the long
+// lines' middle pass) launch one CTA per tile under either policy; their
+// requests for further tiles fail while a kernel of a higher-priority stream
+// waits, so they give way as well: a 32^3 FP32 solve (24 us alone) behind
+// low-priority work takes 60 us behind FP64 256^3 solves, 69 us behind 384^3
+// and 78 us behind FP32 512^3 ones, where kernels with a fixed share of tiles
+// per CTA hold it up for 434, 897 and 1321 us.
 int& launch_grid_mode();
 
 // Per-launch trace for the profiler: an event before the first launch and

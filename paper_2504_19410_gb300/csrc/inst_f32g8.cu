@@ -72,10 +72,12 @@ template <int M> struct Inst8 {
     return e;
   }
   // The C2R pass: X of each solve as a {C, n0 + 1} tensor of 8-byte elements.
-  // The long lines read 64-byte rows; where those lie more than 1.5 MB apart
-  // (each then costs a page translation of its own) generation 2's 256-byte
-  // rows are faster: length 1024 at C = 512^2, 0.434 against 0.488 ms (at C =
-  // 512 x 128 0.116 against 0.079, length 768 at C = 384^2 0.195 against 0.177).
+  // The long lines read 64-byte rows; from a row pitch of about 1.6 MB on,
+  // generation 2's 256-byte rows are faster (why was not measured).  us,
+  // generation 2 / this kernel, GB300:
+  //   C          65,536       98,304        131,072      147,456      196,608      262,144
+  //   M =  768   91.1 / 60.9  133.5 / 94.2  173 / 152    197 / 178    260 / 255    341 / 394
+  //   M = 1024   117 / 78.6   172 / 120     221 / 191    253 / 221    331 / 335    435 / 514
   static constexpr long long kFarRows = 200000;
   template <int NJ> static cudaError_t c2r_n(const Jobs& jobs, long long C, cudaStream_t s) {
     if (WIDE && C > kFarRows) return pass_fns(kArithF32G2, M).c2r(jobs, C, s);

@@ -281,18 +281,17 @@ __global__ void __launch_bounds__(W * T) k_c2r_ax0(const Jobs jobs, long long C)
     // and written by the same thread), then added.
     auto to_sm = [&](int p, V v) { sl.put(p, v); };
     fft_line<P, false, T, V, false, PAD>(t, first, to_sm, sl);
-    using A = typename PairOf<V>::T;
     using IoT = typename Io<V>::T;
     constexpr int NT = W * T, PER = (W * NV + NT - 1) / NT;
     const IoT* rho = static_cast<const IoT*>(jb.aux);
     const IoT beta = ddi_beta<IoT>(jb.par);
     const long long cb = (tile % tpj) * (2 * W);
-    A a[PER];
+    V a[PER];
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
       const int i = threadIdx.x + k * NT, l2 = i % W, p = i / W;
       const long long cc = cb + 2 * l2;
-      a[k] = (p < NV && cc < C) ? load_rho_pair<V>(rho + (long long)p * C + cc) : A{};
+      a[k] = (p < NV && cc < C) ? load_rho_pair<V>(rho + (long long)p * C + cc) : V{};
     }
 #pragma unroll
     for (int k = 0; k < PER; ++k) {

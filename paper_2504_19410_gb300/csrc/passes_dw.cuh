@@ -9,9 +9,12 @@
 //     equal, so in the middle pass the last forward stage leaves a thread
 //     exactly the elements its first inverse stage takes (b + r M/R): the
 //     spectrum multiply happens in registers;
-//   * the first stage's inputs (and the middle pass's spectrum values) are
-//     staged by per-thread asynchronous copies, the next tile's under the
-//     current tile's work, and the twiddles sit in a shared table;
+//   * the first stage's inputs are staged by per-thread asynchronous copies:
+//     in the R2C and row passes the next tile's under the current tile's work,
+//     in the middle pass from its last store on (until then the same slots
+//     hold the spectrum values, copied under the forward transform); the C2R
+//     pass and the plane's middle pass load directly.  The twiddles sit in a
+//     shared table;
 //   * the last stage writes HBM from registers (the row passes too: lanes run
 //     along a row, so their accesses are contiguous), except in the R2C pass,
 //     whose split of two real lines needs each line whole;

@@ -46,8 +46,10 @@
 // q (k_radial_tables) and looked up by the first and the last DCT pass, which
 // saves their per-point evaluation on the FP64 pipe and three passes over
 // the octant.  Measured (GB300, FP64 plan of 256^3): octant
-// 2.60 and spectrum 0.89 ms before, 0.11 ms for the tables now; with the
-// pruned DCT passes the whole generation 6.65 -> 2.00 ms.
+// 2.60 and spectrum 0.89 ms before, 0.046 ms for the tables now (0.107 with
+// the two functions inlined into the table kernel); with the pruned DCT passes
+// the whole generation 6.65 -> 1.95 ms, 6.27 -> 1.99 through the public call
+// with the spectrum copied out.
 // Where there is no memory for a table (a serving plan's W) the same function
 // of q is evaluated per point, with the same bits.  Other grids (no common
 // integer ratio, or a table above a quarter of the octant: planes, very flat
@@ -346,8 +348,9 @@ namespace {
 // One DCT pass: the octant in place, from the U table, or to the spectrum.
 template <int M> struct DctInst {
   using P = typename PlanFor<M>::type;
-  // line pairs per CTA; lengths 48 and 64 in CTAs of about one warp: a 32^3
-  // octant's 545 pairs then spread over 137 SMs' FP64 pipes, not 69
+  // line pairs per CTA: 8; lengths 48 and 64 take 4, CTAs of about one warp, so
+  // that a 32^3 octant's 545 pairs spread over 137 SMs' FP64 pipes, not 69
+  // (54.0 -> 53.2 us; measured at 32^3 alone)
   static constexpr int W = M == 48 || M == 64 ? 4 : 8;
   static constexpr int T = threads_per_line<P, W>();
   static constexpr int SM = smem_strided<P, double2, W>();
