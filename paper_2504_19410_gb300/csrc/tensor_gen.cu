@@ -249,10 +249,8 @@ __device__ __noinline__ double radial_W(const RadialW& w, double q) {
   return w.tab ? w_from_table(w.tab, w.panels, w.c * sqrt(q)) : singular_W(w.kernel, w.c * w.c * q, w.eps * w.eps, w.lam);
 }
 
-// RADIAL: through the integer argument, as the table would hold it.
-template <bool RADIAL>
 __global__ void k_t1_octant(double* __restrict__ O, int kernel, int n0, int n1, int n2, double h0, double h1,
-                            double h2, double eps, double lam, RadialArg arg, const __grid_constant__ RadialU u) {
+                            double h2, double eps, double lam) {
   const long long total = (long long)(n0 + 1) * (n1 + 1) * (n2 + 1);
   const double hv = h0 * h1 * h2;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -261,10 +259,6 @@ __global__ void k_t1_octant(double* __restrict__ O, int kernel, int n0, int n1, 
     const long long r01 = i / (n2 + 1);
     const int p1 = (int)(r01 % (n1 + 1));
     const int p0 = (int)(r01 / (n1 + 1));
-    if constexpr (RADIAL) {
-      O[i] = radial_U(u, arg(p0, p1, p2));
-      continue;
-    }
     const double x = p0 * h0, y = p1 * h1, z = p2 * h2;
     const double r = sqrt(x * x + y * y + z * z);
     O[i] = hv * smooth_U(kernel, r, eps, lam);
@@ -303,12 +297,11 @@ __global__ void k_radial_tables(double* __restrict__ tu, long long nu, double* _
   }
 }
 
-template <typename R, bool RADIAL>
+template <typename R>
 __global__ void k_spectrum_finalize(const double* S1, R* S,  // may alias (FP64 plans)
                                     int kernel, int n0, int n1, int n2,
                                     double c0, double c1, double c2, double eps, double lam, double inv_norm,
-                                    const double* __restrict__ wtab, int wpanels, RadialArg arg,
-                                    const __grid_constant__ RadialW rw) {
+                                    const double* __restrict__ wtab, int wpanels) {
   const long long total = (long long)(n0 + 1) * (n1 + 1) * (n2 + 1);
   const double e2 = eps * eps;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
@@ -317,14 +310,33 @@ __global__ void k_spectrum_finalize(const double* S1, R* S,  // may alias (FP64 
     const long long r01 = i / (n2 + 1);
     const int p1 = (int)(r01 % (n1 + 1));
     const int p0 = (int)(r01 / (n1 + 1));
-    if constexpr (RADIAL) {
-      S[i] = (R)((S1[i] + radial_W(rw, arg(p0, p1, p2))) * inv_norm);
-      continue;
-    }
     const double m0 = c0 * p0, m1 = c1 * p1, m2 = c2 * p2;  // mu_j = pi p_j / (2 L_j)
     const double k2 = m0 * m0 + m1 * m1 + m2 * m2;
     const double w = wtab ? w_from_table(wtab, wpanels, sqrt(k2)) : singular_W(kernel, k2, e2, lam);
     S[i] = (R)((S1[i] + w) * inv_norm);
+  }
+}
+
+// k_t1_octant and k_spectrum_finalize through the integer argument, as the tables
+// would hold it.
+__global__ void k_t1_radial(double* __restrict__ O, int n0, int n1, int n2, RadialArg arg,
+                            const __grid_constant__ RadialU u) {
+  const long long total = (long long)(n0 + 1) * (n1 + 1) * (n2 + 1);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long r01 = i / (n2 + 1);
+    O[i] = radial_U(u, arg((int)(r01 / (n1 + 1)), (int)(r01 % (n1 + 1)), (int)(i % (n2 + 1))));
+  }
+}
+template <typename R>
+__global__ void k_finalize_radial(const double* S1, R* S,  // may alias (FP64 plans)
+                                  int n0, int n1, int n2, double inv_norm, RadialArg arg,
+                                  const __grid_constant__ RadialW w) {
+  const long long total = (long long)(n0 + 1) * (n1 + 1) * (n2 + 1);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long r01 = i / (n2 + 1);
+    S[i] = (R)((S1[i] + radial_W(w, arg((int)(r01 / (n1 + 1)), (int)(r01 % (n1 + 1)), (int)(i % (n2 + 1))))) * inv_norm);
   }
 }
 
@@ -434,16 +446,15 @@ namespace {
 void radial_args(const int n[3], const double L[3], Radial* u, Radial* w) {
   const double pi = 3.14159265358979323846;
   const long long total = (long long)(n[0] + 1) * (n[1] + 1) * (n[2] + 1);
-  double hs[3], cs[3];
-  long double hx[3], cx[3];
+  double hs[3], cs[3], N[3];
+  const double one[3] = {1.0, 1.0, 1.0};
   for (int j = 0; j < 3; ++j) {
     hs[j] = 2.0 * L[j] / n[j];
     cs[j] = pi / (2 * L[j]);
-    hx[j] = (long double)L[j] / n[j];
-    cx[j] = 1.0L / L[j];
+    N[j] = n[j];
   }
-  if (!radial_of(hs, hx, n, total, u)) *u = Radial{};
-  if (!radial_of(cs, cx, n, total, w)) *w = Radial{};
+  if (!radial_of(hs, L, N, n, total, u)) *u = Radial{};
+  if (!radial_of(cs, one, L, n, total, w)) *w = Radial{};
 }
 }  // namespace
 
@@ -488,8 +499,8 @@ cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], 
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && !tu) {
-    (hu ? k_t1_octant<true> : k_t1_octant<false>)<<<blocks_for(total), threads, 0, s>>>(
-        O, (int)kernel, n0, n1, n2, h0, h1, h2, eps, lam, au, fu);
+    if (hu) k_t1_radial<<<blocks_for(total), threads, 0, s>>>(O, n0, n1, n2, au, fu);
+    else k_t1_octant<<<blocks_for(total), threads, 0, s>>>(O, (int)kernel, n0, n1, n2, h0, h1, h2, eps, lam);
     e = cudaGetLastError();
   }
   // axis 2: lines (p0, p1), element stride 1
@@ -508,12 +519,17 @@ cudaError_t tensorgen_run(fsa_kernel kernel, const int n[3], const double L[3], 
         : dtype == FSA_F64 ? dct_run(2 * n0, x0, DctSpectrum<double>{(double*)out, x0, w0, inv_norm}, e1 * e2, e2, s)
                            : dct_run(2 * n0, x0, DctSpectrum<float>{(float*)out, x0, w0, inv_norm}, e1 * e2, e2, s);
   if (e != cudaSuccess || tw) return e;
-  auto finalize = [&](auto kern, auto* S) {
-    kern<<<blocks_for(total), threads, 0, s>>>(O, S, (int)kernel, n0, n1, n2, pi / (2 * L[0]), pi / (2 * L[1]), c2, eps, lam, inv_norm, wtab,
-                                               wtab_panels, aw, fw);
+  auto finalize = [&](auto* S) {
+    using R = std::remove_pointer_t<decltype(S)>;
+    if (hw)
+      k_finalize_radial<R><<<blocks_for(total), threads, 0, s>>>(O, S, n0, n1, n2, inv_norm, aw, fw);
+    else
+      k_spectrum_finalize<R><<<blocks_for(total), threads, 0, s>>>(O, S, (int)kernel, n0, n1, n2, pi / (2 * L[0]),
+                                                                   pi / (2 * L[1]), c2, eps, lam, inv_norm, wtab,
+                                                                   wtab_panels);
   };
-  if (dtype == FSA_F64) finalize(hw ? k_spectrum_finalize<double, true> : k_spectrum_finalize<double, false>, (double*)out);
-  else finalize(hw ? k_spectrum_finalize<float, true> : k_spectrum_finalize<float, false>, (float*)out);
+  if (dtype == FSA_F64) finalize((double*)out);
+  else finalize((float*)out);
   return cudaGetLastError();
 }
 

@@ -12,15 +12,15 @@ int main() {
   double L[3];
   char kind;
   while (std::scanf("%d %d %d %la %la %la %c", n, n + 1, n + 2, L, L + 1, L + 2, &kind) == 7) {
-    double s[3];
-    long double x[3];
+    double s[3], num[3], den[3];
     for (int j = 0; j < 3; ++j) {
       s[j] = kind == 'h' ? 2.0 * L[j] / n[j] : 3.14159265358979323846 / (2 * L[j]);
-      x[j] = kind == 'h' ? (long double)L[j] / n[j] : 1.0L / L[j];
+      num[j] = kind == 'h' ? L[j] : 1.0;
+      den[j] = kind == 'h' ? n[j] : L[j];
     }
     fsa::Radial r{};
     const long long total = (long long)(n[0] + 1) * (n[1] + 1) * (n[2] + 1);
-    if (!fsa::radial_of(s, x, n, total, &r)) {
+    if (!fsa::radial_of(s, num, den, n, total, &r)) {
       std::puts("no");
       continue;
     }
